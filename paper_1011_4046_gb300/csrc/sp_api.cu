@@ -82,7 +82,7 @@ struct SweepGraph {
     int sim = -1;
     int64_t steps = -1, first_local = -1;
     const void *coef = nullptr;
-    const void *phi = nullptr, *tmp = nullptr;
+    const void *phi = nullptr, *tmp = nullptr, *tmp_pc = nullptr;  // tmp_pc: null for single levels
 };
 
 // What the autotuner of the last sp_region_plan measured.
@@ -217,6 +217,8 @@ struct sp_grid {
     size_t cap_trace = 0;
     float2 *d_tmp = nullptr;
     size_t cap_tmp = 0;
+    float4 *d_tmp_pc = nullptr;  // two-level sweep passes only
+    size_t cap_tmp_pc = 0;
     double *d_epart = nullptr, *d_eout = nullptr;
     size_t cap_epart = 0;
     unsigned long long *d_wcount = nullptr;
@@ -675,20 +677,53 @@ int collect_device_error(sp_grid *g)
     return SP_OK;
 }
 
-int enqueue_sweep(sp_grid *g, int s, int64_t nsteps, int64_t first_local, const sp::LevelCoef *d_coef_sim)
+// Whole-grid steps of simulation s.  With a scratch copy of (pi, c) beside
+// that of phi, two levels at a time (launch_columns), else level by level.
+// Level pairs move both arrays to the other copy, single levels only phi, so
+// an even number of pairs leaves (pi, c) in the caller's array and phi needs
+// a copy back after an odd number of single levels, as without pairs.
+int enqueue_sweep(sp_grid *g, int s, int64_t nsteps, int64_t first_local, const sp::LevelCoef *d_coef_sim, bool pairs)
 {
     const sp_params &p = g->p[s];
     const int64_t sites = sites_of(p);
     const sp::PhysConst q = phys_const(p);
     float2 *a = g->phi[s], *b = g->d_tmp;
+    float4 *pa = g->pc[s], *pb = g->d_tmp_pc;
+    const int64_t n_pairs = pairs ? nsteps / 4 * 2 : 0;
     cudaError_t e = cudaSuccess;
-    for (int64_t k = 0; k < nsteps && e == cudaSuccess; ++k) {
-        e = sp::launch_sweep(a, b, g->pc[s], p.n, d_coef_sim, (int)(first_local + k), q, g->stream);
+    int64_t k = 0;
+    for (; k < 2 * n_pairs && e == cudaSuccess; k += 2) {
+        e = sp::launch_columns(a, pa, b, pb, p.n, d_coef_sim + first_local + k, q, g->sm_count, g->stream);
+        std::swap(a, b);
+        std::swap(pa, pb);
+    }
+    for (; k < nsteps && e == cudaSuccess; ++k) {
+        e = sp::launch_sweep(a, b, pa, p.n, d_coef_sim, (int)(first_local + k), q, g->stream);
         std::swap(a, b);
     }
     if (e == cudaSuccess && a != g->phi[s])
         e = cudaMemcpyAsync(g->phi[s], a, sites * sizeof(float2), cudaMemcpyDeviceToDevice, g->stream);
     return e == cudaSuccess ? SP_OK : SP_ECUDA;
+}
+
+// Whether the steps of a sweep call go two levels at a time: from four steps
+// on (fewer hold no even number of pairs), where the state and its phi copy
+// (32 B a site) no longer sit in L2 (measured per level, one at a time / two:
+// 96^3 6.3 / 7.6 us, 128^3 11.4 / 13.2, 144^3 22.5 / 17.1, 160^3 35.2 / 20.9,
+// 256^3 133 / 71, 400^3 509 / 257; 2.5e6 sites are 80 MB), and where the
+// second copy of (pi, c) leaves a sixteenth of the device memory free.
+bool sweep_by_pairs(sp_grid *g, int s, int64_t nsteps)
+{
+    const size_t sites = (size_t)sites_of(g->p[s]);
+    if (nsteps < 4 || sites < 2500000) return false;
+    if (g->d_tmp_pc && g->cap_tmp_pc >= sites) return true;
+    size_t free_b = 0, total_b = 0;
+    if (cudaMemGetInfo(&free_b, &total_b) != cudaSuccess) return false;
+    free_b += g->cap_tmp_pc * sizeof(float4);  // grow() frees the smaller copy first
+    if (free_b < sites * sizeof(float4) + total_b / 16) return false;
+    if (grow(&g->d_tmp_pc, &g->cap_tmp_pc, sites) == cudaSuccess) return true;
+    cudaGetLastError();  // the one-level path needs no such copy
+    return false;
 }
 
 // nsteps whole-grid steps of simulation s.  On a capturable stream the steps
@@ -701,16 +736,17 @@ int sweep_steps(sp_grid *g, int s, int64_t nsteps, int64_t first_local, const sp
     const int64_t sites = sites_of(g->p[s]);
     cudaError_t e = grow(&g->d_tmp, &g->cap_tmp, (size_t)sites);
     if (e != cudaSuccess) return SP_ENOMEM;
-    if (g->stream == nullptr) return enqueue_sweep(g, s, nsteps, first_local, d_coef_sim);
+    const bool pairs = sweep_by_pairs(g, s, nsteps);
+    if (g->stream == nullptr) return enqueue_sweep(g, s, nsteps, first_local, d_coef_sim, pairs);
     SweepGraph &sg = g->sweep_graph;
     if (!(sg.exec && sg.sim == s && sg.steps == nsteps && sg.first_local == first_local && sg.coef == d_coef_sim &&
-          sg.phi == g->phi[s] && sg.tmp == g->d_tmp)) {
+          sg.phi == g->phi[s] && sg.tmp == g->d_tmp && sg.tmp_pc == (pairs ? g->d_tmp_pc : nullptr))) {
         if (sg.exec) cudaGraphExecDestroy(sg.exec);
         sg.exec = nullptr;
         cudaGraph_t graph = nullptr;
         e = cudaStreamBeginCapture(g->stream, cudaStreamCaptureModeThreadLocal);
         if (e != cudaSuccess) return SP_ECUDA;
-        int rc = enqueue_sweep(g, s, nsteps, first_local, d_coef_sim);
+        int rc = enqueue_sweep(g, s, nsteps, first_local, d_coef_sim, pairs);
         e = cudaStreamEndCapture(g->stream, &graph);
         if (rc != SP_OK || e != cudaSuccess) {
             if (graph) cudaGraphDestroy(graph);
@@ -728,6 +764,7 @@ int sweep_steps(sp_grid *g, int s, int64_t nsteps, int64_t first_local, const sp
         sg.coef = d_coef_sim;
         sg.phi = g->phi[s];
         sg.tmp = g->d_tmp;
+        sg.tmp_pc = pairs ? g->d_tmp_pc : nullptr;
     }
     return cudaGraphLaunch(sg.exec, g->stream) == cudaSuccess ? SP_OK : SP_ECUDA;
 }
@@ -771,7 +808,7 @@ int enqueue_region_call(sp_grid *g, const std::vector<GroupLaunch> &groups, int6
         const int H = g->B[s] / 2;
         const int64_t done = (n_steps / H) * H;
         if (n_steps - done <= 0) continue;
-        const int rc = enqueue_sweep(g, s, n_steps - done, done, g->d_coef + (size_t)s * n_steps);
+        const int rc = enqueue_sweep(g, s, n_steps - done, done, g->d_coef + (size_t)s * n_steps, false);
         if (rc != SP_OK) return rc;
     }
     return SP_OK;
@@ -1963,6 +2000,7 @@ int sp_destroy(sp_grid *g)
     cudaFree(g->d_coef);
     cudaFree(g->d_trace);
     cudaFree(g->d_tmp);
+    cudaFree(g->d_tmp_pc);
     cudaFree(g->d_epart);
     cudaFree(g->d_eout);
     cudaFree(g->d_wcount);

@@ -15,6 +15,10 @@ cudaError_t region_occupancy(int threads, int B, size_t smem, int *blocks_per_sm
 cudaError_t launch_region(const RegionArgs &a, int threads, int max_B, size_t smem, int grid, cudaStream_t st);
 cudaError_t launch_sweep(const float2 *phi_in, float2 *phi_out, float4 *pc, const int n[3],
                          const LevelCoef *coef, int lvl, PhysConst q, cudaStream_t st);
+// Two levels of the whole grid in one pass, from one copy of the state to
+// another (sp_columns.cu); coef: of the first of them.
+cudaError_t launch_columns(const float2 *phi_in, const float4 *pc_in, float2 *phi_out, float4 *pc_out, const int n[3],
+                           const LevelCoef *coef, PhysConst q, int sm_count, cudaStream_t st);
 int energy_blocks(const int n[3]);
 cudaError_t launch_energy(const float2 *phi, const float4 *pc, const int n[3], double inv_dx2, double eta2,
                           double half_lambda_a2, double *partial, double *out, cudaStream_t st);
