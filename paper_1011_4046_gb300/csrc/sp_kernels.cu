@@ -621,15 +621,20 @@ __global__ void __launch_bounds__(NW + 32, region_min_blocks(NW)) region_kernel(
 }
 
 // ------------------------------------------------------------ sweep kernel
-// One level of the whole grid: block 32 x 8 over (x, y), each thread marches
+// One level of the whole grid: block 32 x 4 over (x, y), each thread marches
 // a chunk of z keeping phi(z-1), phi(z), phi(z+1) in registers; x and y
-// neighbours come through L1.  48 bytes per site-update of HBM traffic.
-__global__ void __launch_bounds__(256) sweep_kernel(const float2 *__restrict__ phi_in, float2 *__restrict__ phi_out,
-                                                    float4 *__restrict__ pc, int nx, int ny, int nz, int zchunk,
-                                                    const LevelCoef *__restrict__ coef, int lvl, PhysConst q)
+// neighbours come through L1.  48 bytes per site-update: bound by DRAM beyond
+// L2, by L2 and the chain of its round trips below.  Ten blocks of 128 threads
+// per SM (48 registers): 512 x 512 x 128 249.5 us, 128^3 10.7 us; the same
+// threads as five blocks of 32 x 8 253.4 and 11.0 us, and at 40 registers, six
+// blocks, 259 and 12.0 us.
+constexpr int kSweepY = 4, kSweepPerSm = 10;
+__global__ void __launch_bounds__(32 * kSweepY, kSweepPerSm)
+    sweep_kernel(const float2 *__restrict__ phi_in, float2 *__restrict__ phi_out, float4 *__restrict__ pc, int nx, int ny,
+                 int nz, int zchunk, const LevelCoef *__restrict__ coef, int lvl, PhysConst q)
 {
     const int x = blockIdx.x * 32 + threadIdx.x;
-    const int y = blockIdx.y * 8 + threadIdx.y;
+    const int y = blockIdx.y * kSweepY + threadIdx.y;
     if (x >= nx || y >= ny) return;
     const int z0 = blockIdx.z * zchunk;
     const int z1 = min(z0 + zchunk, nz);
@@ -962,9 +967,20 @@ cudaError_t launch_region(const RegionArgs &a, int threads, int max_B, size_t sm
 cudaError_t launch_sweep(const float2 *phi_in, float2 *phi_out, float4 *pc, const int n[3],
                          const LevelCoef *coef, int lvl, PhysConst q, cudaStream_t st)
 {
-    const int zchunk = 8;
-    dim3 block(32, 8, 1);
-    dim3 grid((n[0] + 31) / 32, (n[1] + 7) / 8, (n[2] + zchunk - 1) / zchunk);
+    // Planes a block marches through.  A grid of few blocks takes one plane
+    // per block (the march is a chain of L2 round trips: 48 x 40 x 36 takes 3.93
+    // us a level at eight planes, 1.81 at one), and more as that makes one full
+    // wave of resident blocks (64^3: 4.14 us at eight planes, 2.86 at two).
+    // Beyond six planes a wave, chunks of four keep the last wave small (150 x
+    // 77 x 131: 10.4 us at eight planes, 9.1 at four; 128^3: 11.4 and 10.7),
+    // until the waves are so many that the two extra planes a chunk reads weigh
+    // more (512 x 512 x 128: 249.5 us at eight, 249.9 at four).
+    const dim3 block(32, kSweepY, 1);
+    dim3 grid((n[0] + 31) / 32, (n[1] + kSweepY - 1) / kSweepY, 1);
+    constexpr long long kWave = 152ll * kSweepPerSm;
+    const long long waves = ((long long)grid.x * grid.y * n[2] + kWave - 1) / kWave;
+    const int zchunk = waves <= 6 ? (int)waves : waves <= 64 ? 4 : 8;
+    grid.z = (n[2] + zchunk - 1) / zchunk;
     sweep_kernel<<<grid, block, 0, st>>>(phi_in, phi_out, pc, n[0], n[1], n[2], zchunk, coef, lvl, q);
     return cudaGetLastError();
 }
