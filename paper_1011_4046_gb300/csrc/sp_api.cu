@@ -219,9 +219,9 @@ struct sp_grid {
     size_t cap_tmp = 0;
     float4 *d_tmp_pc = nullptr;  // two-level sweep passes only
     size_t cap_tmp_pc = 0;
-    double *d_epart = nullptr, *d_eout = nullptr;
+    char *d_epart = nullptr;  // diagnostics: sums per block, and the result
     size_t cap_epart = 0;
-    unsigned long long *d_wcount = nullptr;
+    sp::DiagOut *d_diag = nullptr;
     signed char *d_wind = nullptr;
     size_t cap_wind = 0;
     // last region launch
@@ -1495,8 +1495,7 @@ int sp_grid_create(const sp_params *p, int32_t n_sims, void *const *state_dev, v
     }
     e = cudaMalloc((void **)&g->d_ctl, kMaxGroups * sizeof(sp::Ctl));
     if (e == cudaSuccess) e = cudaMemsetAsync(g->d_ctl, 0, kMaxGroups * sizeof(sp::Ctl), g->stream);
-    if (e == cudaSuccess) e = cudaMalloc((void **)&g->d_eout, 4 * sizeof(double));
-    if (e == cudaSuccess) e = cudaMalloc((void **)&g->d_wcount, 8 * sizeof(unsigned long long));
+    if (e == cudaSuccess) e = cudaMalloc((void **)&g->d_diag, sizeof(sp::DiagOut));
     if (e != cudaSuccess) {
         sp_destroy(g);
         return SP_ENOMEM;
@@ -1827,8 +1826,7 @@ int sp_read_surface(const sp_grid *gc, int32_t sim, int32_t what, void *dst, siz
             if (e != cudaSuccess) return SP_ENOMEM;
             w = g->d_wind;
         }
-        e = cudaMemsetAsync(g->d_wcount, 0, 8 * sizeof(unsigned long long), g->stream);
-        if (e == cudaSuccess) e = sp::launch_winding(g->phi[sim], p.n, w, g->d_wcount, g->stream);
+        e = sp::launch_winding_map(g->phi[sim], p.n, w, g->stream);
         if (e == cudaSuccess && !dst_is_device)
             e = cudaMemcpyAsync(dst, w, (size_t)(3 * sites), cudaMemcpyDeviceToHost, g->stream);
         if (e == cudaSuccess) e = cudaStreamSynchronize(g->stream);
@@ -1836,19 +1834,14 @@ int sp_read_surface(const sp_grid *gc, int32_t sim, int32_t what, void *dst, siz
     }
     case SP_SURF_DIAG: {
         if (dst_bytes < sizeof(sp_diag)) return SP_EINVAL;
-        const int nb = sp::energy_blocks(p.n);
-        e = grow(&g->d_epart, &g->cap_epart, (size_t)3 * nb);
+        e = grow(&g->d_epart, &g->cap_epart, sp::diag_scratch_bytes(p.n));
         if (e != cudaSuccess) return SP_ENOMEM;
         double tau, a, d;
         level_physics(p, g->level[sim], &tau, &a, &d);
-        e = sp::launch_energy(g->phi[sim], g->pc[sim], p.n, 1.0 / (p.dx * p.dx), p.eta * p.eta,
-                              0.5 * p.lambda * a * a, g->d_epart, g->d_eout, g->stream);
-        if (e == cudaSuccess) e = cudaMemsetAsync(g->d_wcount, 0, 8 * sizeof(unsigned long long), g->stream);
-        if (e == cudaSuccess) e = sp::launch_winding(g->phi[sim], p.n, nullptr, g->d_wcount, g->stream);
-        double en[3];
-        unsigned long long wc[7];
-        if (e == cudaSuccess) e = cudaMemcpyAsync(en, g->d_eout, sizeof en, cudaMemcpyDeviceToHost, g->stream);
-        if (e == cudaSuccess) e = cudaMemcpyAsync(wc, g->d_wcount, sizeof wc, cudaMemcpyDeviceToHost, g->stream);
+        e = sp::launch_diag(g->phi[sim], g->pc[sim], p.n, 1.0 / (p.dx * p.dx), p.eta * p.eta, 0.5 * p.lambda * a * a,
+                            g->d_epart, g->d_diag, g->stream);
+        sp::DiagOut r;
+        if (e == cudaSuccess) e = cudaMemcpyAsync(&r, g->d_diag, sizeof r, cudaMemcpyDeviceToHost, g->stream);
         if (e == cudaSuccess) e = cudaStreamSynchronize(g->stream);
         if (e != cudaSuccess) return SP_ECUDA;
         sp_diag out;
@@ -1856,16 +1849,16 @@ int sp_read_surface(const sp_grid *gc, int32_t sim, int32_t what, void *dst, siz
         out.level = g->level[sim];
         out.tau = tau;
         out.a = a;
-        out.kinetic = en[0];
-        out.gradient = en[1];
-        out.potential = en[2];
-        out.total = en[0] + en[1] + en[2];
+        out.kinetic = r.energy[0];
+        out.gradient = r.energy[1];
+        out.potential = r.energy[2];
+        out.total = r.energy[0] + r.energy[1] + r.energy[2];
         for (int k = 0; k < 3; ++k) {
-            out.pierced[k] = (int64_t)wc[k];
-            out.net_winding[k] = (int64_t)wc[4 + k];
+            out.pierced[k] = r.winding[k];
+            out.net_winding[k] = r.winding[4 + k];
         }
-        out.abs_winding = (int64_t)wc[3];
-        out.string_length = (double)(wc[0] + wc[1] + wc[2]) * p.dx;
+        out.abs_winding = r.winding[3];
+        out.string_length = (double)(r.winding[0] + r.winding[1] + r.winding[2]) * p.dx;
         if (dst_is_device) e = cudaMemcpy(dst, &out, sizeof out, cudaMemcpyHostToDevice);
         else std::memcpy(dst, &out, sizeof out);
         return cuda_err(e);
@@ -2002,8 +1995,7 @@ int sp_destroy(sp_grid *g)
     cudaFree(g->d_tmp);
     cudaFree(g->d_tmp_pc);
     cudaFree(g->d_epart);
-    cudaFree(g->d_eout);
-    cudaFree(g->d_wcount);
+    cudaFree(g->d_diag);
     cudaFree(g->d_wind);
     cudaFree(g->d_feat);
     cudaFree(g->d_simf);

@@ -3,13 +3,13 @@
 //   reset_kernel   arms the dependency counters and seeds the ready queue
 //   region_kernel  persistent: pops ready regions and evolves each on chip
 //   sweep_kernel   monolithic whole-grid step (the comparator)
-//   energy_*       FP64 energy of a stored state (deterministic reduction)
-//   winding_kernel exact per-plaquette winding numbers and string counts
+//   feature_kernel inputs of the region cost model
 //
 // All arithmetic of the evolution goes through sp::site_update (sp_update.h).
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include "sp_crossing.cuh"
 #include "sp_device.cuh"
 #include "sp_kernels.h"
 #include "sp_region_common.cuh"
@@ -661,120 +661,6 @@ __global__ void __launch_bounds__(32 * kSweepY, kSweepPerSm)
     }
 }
 
-// ------------------------------------------------------------ diagnostics
-// Energy terms of a stored state in FP64: sum |pi|^2, sum over forward links
-// |phi(x+e) - phi(x)|^2 / dx^2 and sum a^2 (lambda/2)(|phi|^2 - eta^2)^2.
-// Each block reduces a fixed range of sites in a fixed tree order; the
-// partials are then summed in block order: the result is deterministic.
-constexpr int kDiagThreads = 256;
-
-__global__ void __launch_bounds__(kDiagThreads)
-    energy_partial_kernel(const float2 *__restrict__ phi, const float4 *__restrict__ pc, int nx, int ny, int nz,
-                          double inv_dx2, double eta2, double half_lambda_a2, double *__restrict__ partial)
-{
-    __shared__ double red[3][kDiagThreads];
-    const long long sites = (long long)nx * ny * nz;
-    const long long per_block = (sites + gridDim.x - 1) / gridDim.x;
-    const long long s0 = blockIdx.x * per_block;
-    const long long s1 = min(s0 + per_block, sites);
-    double kin = 0.0, grad = 0.0, pot = 0.0;
-    for (long long s = s0 + threadIdx.x; s < s1; s += kDiagThreads) {
-        const int x = (int)(s % nx);
-        const int y = (int)((s / nx) % ny);
-        const int z = (int)(s / ((long long)nx * ny));
-        const float2 f = phi[s];
-        const float4 v = pc[s];
-        const double fr = f.x, fi = f.y;
-        kin = __dadd_rn(kin, __dadd_rn(__dmul_rn((double)v.x, (double)v.x), __dmul_rn((double)v.y, (double)v.y)));
-        const long long nb[3] = {s - x + (x == nx - 1 ? 0 : x + 1),
-                                 s + (long long)((y == ny - 1 ? 0 : y + 1) - y) * nx,
-                                 s + (long long)((z == nz - 1 ? 0 : z + 1) - z) * nx * ny};
-        for (int k = 0; k < 3; ++k) {
-            const float2 g = phi[nb[k]];
-            const double dr = __dsub_rn((double)g.x, fr), di = __dsub_rn((double)g.y, fi);
-            grad = __dadd_rn(grad, __dmul_rn(__dadd_rn(__dmul_rn(dr, dr), __dmul_rn(di, di)), inv_dx2));
-        }
-        const double m2 = __dsub_rn(__dadd_rn(__dmul_rn(fr, fr), __dmul_rn(fi, fi)), eta2);
-        pot = __dadd_rn(pot, __dmul_rn(half_lambda_a2, __dmul_rn(m2, m2)));
-    }
-    red[0][threadIdx.x] = kin;
-    red[1][threadIdx.x] = grad;
-    red[2][threadIdx.x] = pot;
-    __syncthreads();
-    for (int w = kDiagThreads / 2; w > 0; w >>= 1) {
-        if (threadIdx.x < w)
-            for (int k = 0; k < 3; ++k) red[k][threadIdx.x] = __dadd_rn(red[k][threadIdx.x], red[k][threadIdx.x + w]);
-        __syncthreads();
-    }
-    if (threadIdx.x == 0)
-        for (int k = 0; k < 3; ++k) partial[3 * blockIdx.x + k] = red[k][0];
-}
-
-__global__ void energy_final_kernel(const double *__restrict__ partial, int nblocks, double *__restrict__ out)
-{
-    if (threadIdx.x != 0 || blockIdx.x != 0) return;
-    double acc[3] = {0.0, 0.0, 0.0};
-    for (int b = 0; b < nblocks; ++b)
-        for (int k = 0; k < 3; ++k) acc[k] = __dadd_rn(acc[k], partial[3 * b + k]);
-    for (int k = 0; k < 3; ++k) out[k] = acc[k];
-}
-
-// Winding of the field around each plaquette: signed crossings of the
-// positive real axis by the polygon phi(p0) phi(p1) phi(p2) phi(p3)
-// (corners x, x+e_a, x+e_a+e_b, x+e_b; (a, b) = (k+1, k+2) mod 3).  An edge
-// u -> v crossing upward counts +1 when cross(u, v) >= 0, downward -1 when
-// cross(u, v) <= 0; a vertex on the axis counts as above it.  The products
-// of FP32 inputs are exact in FP64, so the sign tests are exact.
-__device__ __forceinline__ int crossing(float2 u, float2 v)
-{
-    const double cr = __dsub_rn(__dmul_rn((double)u.x, (double)v.y), __dmul_rn((double)u.y, (double)v.x));
-    const bool ua = u.y >= 0.0f, va = v.y >= 0.0f;
-    if (!ua && va) return cr >= 0.0 ? 1 : 0;
-    if (ua && !va) return cr <= 0.0 ? -1 : 0;
-    return 0;
-}
-
-__global__ void __launch_bounds__(kDiagThreads)
-    winding_kernel(const float2 *__restrict__ phi, int nx, int ny, int nz, signed char *__restrict__ w,
-                   unsigned long long *__restrict__ counts)
-{
-    // counts: [0..2] pierced plaquettes per normal axis, [3] sum |w|, [4..6] sum w (two's complement)
-    __shared__ unsigned long long red[7];
-    if (threadIdx.x < 7) red[threadIdx.x] = 0ull;
-    __syncthreads();
-    const long long sites = (long long)nx * ny * nz;
-    unsigned long long loc[7] = {0, 0, 0, 0, 0, 0, 0};
-    for (long long s = (long long)blockIdx.x * blockDim.x + threadIdx.x; s < sites;
-         s += (long long)gridDim.x * blockDim.x) {
-        const int c[3] = {(int)(s % nx), (int)((s / nx) % ny), (int)(s / ((long long)nx * ny))};
-        const int n[3] = {nx, ny, nz};
-        for (int k = 0; k < 3; ++k) {
-            const int a = (k + 1) % 3, b = (k + 2) % 3;
-            int q1[3] = {c[0], c[1], c[2]}, q2[3] = {c[0], c[1], c[2]}, q3[3] = {c[0], c[1], c[2]};
-            q1[a] = q1[a] + 1 == n[a] ? 0 : q1[a] + 1;
-            q2[a] = q1[a];
-            q2[b] = q2[b] + 1 == n[b] ? 0 : q2[b] + 1;
-            q3[b] = q2[b];
-            const float2 p0 = phi[s];
-            const float2 p1 = phi[q1[0] + (long long)nx * (q1[1] + (long long)ny * q1[2])];
-            const float2 p2 = phi[q2[0] + (long long)nx * (q2[1] + (long long)ny * q2[2])];
-            const float2 p3 = phi[q3[0] + (long long)nx * (q3[1] + (long long)ny * q3[2])];
-            const int tot = crossing(p0, p1) + crossing(p1, p2) + crossing(p2, p3) + crossing(p3, p0);
-            if (w) w[k * sites + s] = (signed char)tot;
-            if (tot != 0) {
-                loc[k] += 1ull;
-                loc[3] += (unsigned long long)(tot < 0 ? -tot : tot);
-                loc[4 + k] += (unsigned long long)(long long)tot;
-            }
-        }
-    }
-    for (int k = 0; k < 7; ++k)
-        if (loc[k]) atomicAdd(&red[k], loc[k]);
-    __syncthreads();
-    if (threadIdx.x < 7 && red[threadIdx.x]) atomicAdd(&counts[threadIdx.x], red[threadIdx.x]);
-}
-
-// ------------------------------------------------------------ launchers
 // ------------------------------------------------------------ region features
 // The 16 inputs of the region cost model, per region of a launch, from its
 // descriptor and from the state at the start of the call (the footprint of
@@ -982,33 +868,6 @@ cudaError_t launch_sweep(const float2 *phi_in, float2 *phi_out, float4 *pc, cons
     const int zchunk = waves <= 6 ? (int)waves : waves <= 64 ? 4 : 8;
     grid.z = (n[2] + zchunk - 1) / zchunk;
     sweep_kernel<<<grid, block, 0, st>>>(phi_in, phi_out, pc, n[0], n[1], n[2], zchunk, coef, lvl, q);
-    return cudaGetLastError();
-}
-
-int energy_blocks(const int n[3])
-{
-    const long long sites = (long long)n[0] * n[1] * n[2];
-    long long b = (sites + 4095) / 4096;
-    return (int)(b < 1 ? 1 : (b > 4096 ? 4096 : b));
-}
-
-cudaError_t launch_energy(const float2 *phi, const float4 *pc, const int n[3], double inv_dx2, double eta2,
-                          double half_lambda_a2, double *partial, double *out, cudaStream_t st)
-{
-    const int nb = energy_blocks(n);
-    energy_partial_kernel<<<nb, kDiagThreads, 0, st>>>(phi, pc, n[0], n[1], n[2], inv_dx2, eta2, half_lambda_a2,
-                                                        partial);
-    energy_final_kernel<<<1, 32, 0, st>>>(partial, nb, out);
-    return cudaGetLastError();
-}
-
-cudaError_t launch_winding(const float2 *phi, const int n[3], signed char *w, unsigned long long *counts,
-                           cudaStream_t st)
-{
-    const long long sites = (long long)n[0] * n[1] * n[2];
-    long long b = (sites + kDiagThreads - 1) / kDiagThreads;
-    if (b > 8192) b = 8192;
-    winding_kernel<<<(int)b, kDiagThreads, 0, st>>>(phi, n[0], n[1], n[2], w, counts);
     return cudaGetLastError();
 }
 

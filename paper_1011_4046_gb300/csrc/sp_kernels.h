@@ -19,11 +19,16 @@ cudaError_t launch_sweep(const float2 *phi_in, float2 *phi_out, float4 *pc, cons
 // another (sp_columns.cu); coef: of the first of them.
 cudaError_t launch_columns(const float2 *phi_in, const float4 *pc_in, float2 *phi_out, float4 *pc_out, const int n[3],
                            const LevelCoef *coef, PhysConst q, int sm_count, cudaStream_t st);
-int energy_blocks(const int n[3]);
-cudaError_t launch_energy(const float2 *phi, const float4 *pc, const int n[3], double inv_dx2, double eta2,
-                          double half_lambda_a2, double *partial, double *out, cudaStream_t st);
-cudaError_t launch_winding(const float2 *phi, const int n[3], signed char *w, unsigned long long *counts,
-                           cudaStream_t st);
+// Diagnostics of a stored state (sp_diag.cu): energy terms and winding counts
+// in one pass, and the map of plaquette windings [3][sites].
+struct DiagOut {
+    double energy[3];      // kinetic, gradient, potential
+    long long winding[7];  // pierced plaquettes by normal axis, sum |w|, sum w by normal axis
+};
+size_t diag_scratch_bytes(const int n[3]);
+cudaError_t launch_diag(const float2 *phi, const float4 *pc, const int n[3], double inv_dx2, double eta2,
+                        double half_lambda_a2, void *scratch, DiagOut *out, cudaStream_t st);
+cudaError_t launch_winding_map(const float2 *phi, const int n[3], signed char *map, cudaStream_t st);
 
 }  // namespace sp
 
