@@ -168,7 +168,8 @@ typedef struct {
     double tune_best_ms;     /* its trial time of the chosen candidate (16 steps) */
     double tune_default_ms;  /* its trial time of the default choice, 0 if not timed */
     int32_t mailbox_slots;   /* 2: ring of two band slots; 1: one slot for every band (0: lattice) */
-    int32_t region_shape;    /* SP_SHAPE_SPLIT or SP_SHAPE_LATTICE; for a lattice plan "band" reads
+    int32_t region_shape;    /* SP_SHAPE_SPLIT or SP_SHAPE_LATTICE; for a lattice plan ctas_per_sm and
+                                grid count the regions resident per SM and in all, "band" reads
                                 "layer" (s levels: 4 M_x M_y M_z regions, N_d = B M_d) and
                                 mailbox_bytes holds the odd-level phi array */
 } sp_plan_info;
@@ -205,8 +206,8 @@ int sp_grid_create(const sp_params *p, int32_t n_sims, void *const *state_dev, v
  *                a multiple of B; 0 takes 16 where it divides, else 8, else
  *                4; SP_AUTOTUNE times the sizes that divide every side.
  *   block_shape: worker threads per CTA (64, 128, 256, 320, 384, 480, 512 or 768;
- *                lattice plans: 64, 128, 192, 256 or 512, one region per CTA
- *                and no manager warp (default: 128 up to s = 4, 256 at
+ *                lattice plans: 64, 128, 192, 256 or 512 per region
+ *                and no manager warp (default: 64 up to s = 3, 128 at s = 4, 256 at
  *                s = 5, 512 at s = 6);
  *                every worker taking every step of a region); one manager
  *                warp is added.  0 for the default of each base (64 for

@@ -284,6 +284,27 @@ std::string build_lattice_tables(int s, LatticeTables *t)
     }
     t->cell_off[K] = (int32_t)t->cell.size();
 
+    // the wide cell entries, where the steps fit
+    {
+        bool fits = t->n_slots <= (int)kLatWideSlotMask + 1;
+        std::vector<uint32_t> wide;
+        for (const uint32_t e : t->cell) {
+            const uint64_t nb = t->row_nb[lat_row(e)];
+            const int step[5] = {lat_dym(nb) + bank_a, lat_dyp(nb) - bank_a, lat_dzm(nb) + bank_b, lat_dzp(nb) - bank_b,
+                                 t->row_pc[lat_row(e)]};
+            uint32_t m[5];
+            for (int i = 0; i < 5; ++i) {
+                if (e && step[i] % 16) return fail("row step off its bank residue");
+                fits = fits && step[i] / 16 >= -128 && step[i] / 16 <= 127;
+                m[i] = (uint32_t)(step[i] / 16) & 0xffu;
+            }
+            wide.push_back((uint32_t)lat_slot(e) | (uint32_t)lat_row(e) << kLatWideRowShift |
+                           ((e & kLatExpPhi) ? kLatWideExpPhi : 0u) | ((e & kLatExpPc) ? kLatWideExpPc : 0u) | m[4] << 24);
+            wide.push_back(m[0] | m[1] << 8 | m[2] << 16 | m[3] << 24);
+        }
+        if (fits) t->cell_wide = wide;
+    }
+
     // imports before level k: full (cells entering), phi only (neighbours outside)
     t->imp_off.assign(K + 1, 0);
     t->imp_n.assign(K, 0);
@@ -344,6 +365,34 @@ std::string build_lattice_tables(int s, LatticeTables *t)
         std::sort(all.begin(), all.end());
         for (const auto &x : all) t->imp_all.push_back(x.second.first), t->imp_all.push_back(x.second.second);
     }
+    {
+        // imp_run: an entry per import, or, where every slot has the parity of
+        // its site, per pair of imports in an even slot and the next one that
+        // are x neighbours of one row
+        const bool parity = (bank_a | bank_b) % 2 == 0;
+        std::map<std::pair<int, int>, size_t> at;  // (slot, buffer) -> index in imp_all
+        auto key = [&](size_t i) { return std::make_pair(lat_slot(t->imp_all[i]), (t->imp_all[i] & kLatImpBuf) ? 1 : 0); };
+        for (size_t i = 0; i < t->imp_all.size(); i += 2) at[key(i)] = i;
+        size_t imports = 0;
+        for (size_t i = 0; i < t->imp_all.size(); i += 2) {
+            const uint32_t e = t->imp_all[i], k = t->imp_all[i + 1];
+            const auto other = at.find({lat_slot(e) ^ 1, key(i).second});
+            const bool pair = parity && (e & kLatImpPairRow) && other != at.end();
+            if (pair && (lat_slot(e) & 1)) continue;  // in its lower neighbour's entry
+            uint32_t w = k | k << 8;
+            if (pair) {
+                const uint32_t e2 = t->imp_all[other->second], k2 = t->imp_all[other->second + 1];
+                if (lat_row(e2) != lat_row(e) || lat_rx2s(e2) != lat_rx2s(e) + 1) return fail("pair of imports not x neighbours");
+                w = std::min(k, k2) | std::max(k, k2) << 8 | kLatRunPair | ((e2 & kLatImpFull) ? kLatRunFull2 : 0u);
+            }
+            t->imp_run.push_back(e);
+            t->imp_run.push_back(w | (uint32_t)t->row_pc[lat_row(e)] << kLatRunPcShift);
+            if (lat_run_pc(t->imp_run.back()) != t->row_pc[lat_row(e)]) return fail("(pi, c) step of an import beyond 14 bits");
+            imports += pair ? 2 : 1;
+            t->run_pairs = t->run_pairs || pair;
+        }
+        if (2 * imports != t->imp_all.size()) return fail("imports lost between the two lists");
+    }
     t->bytes_read = 24 * t->imports_full + 8 * t->imports_phi;
     t->bytes_written = 8 * t->exports_phi + 16 * t->exports_pc;
 
@@ -375,6 +424,22 @@ std::string build_lattice_tables(int s, LatticeTables *t)
             if (!x_ok(t->cell[i])) return fail("cell entry with a wrong x field (level %d)", k);
         for (int i = t->imp_off[k]; i < t->imp_off[k] + t->imp_n[k]; ++i)
             if (!x_ok(t->imp[i])) return fail("import entry with a wrong x field (level %d)", k);
+    }
+    // check 0b: the wide entries give the same slot, row, flags, neighbour slots
+    // and (pi, c) index as the narrow ones
+    for (size_t i = 0; 2 * i < t->cell_wide.size(); ++i) {
+        const uint32_t e = t->cell[i], w0 = t->cell_wide[2 * i], w1 = t->cell_wide[2 * i + 1];
+        if (!e) continue;  // padding
+        R3 r;
+        int nb[7], pc;
+        decode(e, &r, nb, &pc);
+        const int sl = (int)(w0 & kLatWideSlotMask);
+        auto step = [](uint32_t w, int byte) { return 16 * (int)(int8_t)(uint8_t)(w >> (8 * byte) & 0xffu); };
+        if (sl != nb[0] || (int)((w0 >> kLatWideRowShift) & kLatRowMask) != lat_row(e) ||
+            ((w0 & kLatWideExpPhi) != 0) != ((e & kLatExpPhi) != 0) || ((w0 & kLatWideExpPc) != 0) != ((e & kLatExpPc) != 0) ||
+            sl + step(w0, 3) != pc || sl - bank_a + step(w1, 0) != nb[3] || sl + bank_a + step(w1, 1) != nb[4] ||
+            sl - bank_b + step(w1, 2) != nb[5] || sl + bank_b + step(w1, 3) != nb[6])
+            return fail("wide cell entry %d differs from the narrow one", (int)i);
     }
     // check 1: entries decode to their cells, and every value level k reads
     // is computed at level k - 1 or imported before level k

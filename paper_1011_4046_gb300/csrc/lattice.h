@@ -98,6 +98,22 @@ constexpr int kLatMaxS = 6;  // slot indices are 13 bits, coordinates 5 bits per
 // all its imports at its start: imp_all holds them in one list, sorted by
 // buffer and by offset from the centre (z, y, x: ascending addresses), each
 // with its level, which regions cut by a call's first or last level filter.
+// imp_run is what the kernel reads: imp_all with the two imports of an aligned
+// slot pair (an even slot and its neighbour in x, same row and buffer) as one
+// entry, 1370 instead of 2437 at s = 4.  An entry is the lower import's word
+// and a second word: the first and last level of its imports (bits 0..7 and
+// 8..15), for a pair whether the upper one is full (bit 16) and bit 17, and
+// the (pi, c) index minus the slot (bits 18..31, signed; x neighbours share it).
+// A region cut by the call's first or last level loads an entry when any of
+// its levels is the region's; the other half then gets the bytes of its
+// own site, which are what any load of that slot writes, or is not used.
+// cell_wide holds the cell entries for the kernel that keeps the whole list in
+// shared memory, with what a cell needs of its row: as slots, and (pi, c)
+// indices, are congruent to x + a y + b z mod 16, the steps to the y and z
+// neighbours and to the (pi, c) index are -a, a, -b, b and 0 plus multiples of
+// 16, which fit a signed byte up to s = 5 (cell_wide is empty beyond).  Word 0:
+// slot (bits 0..11), row (12..21), export phi (22), export (pi, c) (23), (pi, c)
+// step / 16 (24..31); word 1: the four neighbours' multiples, y - 1 lowest.
 // Every level's lists start on a 16-byte boundary (padded with zero entries
 // to a multiple of four).
 constexpr uint32_t kLatSlotMask = 0x1fffu;
@@ -119,6 +135,16 @@ constexpr uint32_t kLatImpPair = 1u << 30;
 // neighbour writes the partner slot the same bytes any other load of it
 // does, so such a region may copy the pairs with this bit.
 constexpr uint32_t kLatImpPairRow = 1u << 31;
+constexpr uint32_t kLatRunFull2 = 1u << 16;  // second word of imp_run: the upper import of the pair is full
+constexpr uint32_t kLatRunPair = 1u << 17;   // the entry holds a pair of imports
+constexpr int kLatRunPcShift = 18;
+constexpr uint32_t kLatWideSlotMask = 0xfffu;
+constexpr int kLatWideRowShift = 12;
+constexpr uint32_t kLatWideExpPhi = 1u << 22;
+constexpr uint32_t kLatWideExpPc = 1u << 23;
+LAT_HD int lat_run_pc(uint32_t w) { return (int)w >> kLatRunPcShift; }
+LAT_HD int lat_run_first(uint32_t w) { return (int)(w & 0xffu); }
+LAT_HD int lat_run_last(uint32_t w) { return (int)((w >> 8) & 0xffu); }
 constexpr int kLatRxShift = 25;
 constexpr uint32_t kLatRxMask = 0x1fu;  // 4s <= 24
 
@@ -146,10 +172,13 @@ struct LatticeTables {
     std::vector<uint32_t> row_xy;   // rb_side^2
     int bank_a = 0, bank_b = 0;     // slot residue rx + a ry + b rz mod 16
     std::vector<uint32_t> cell;     // level k: cell[cell_off[k] .. cell_off[k] + cell_n[k]), padded
+    std::vector<uint32_t> cell_wide;  // two words per entry of cell, or empty
     std::vector<int32_t> cell_off, cell_n;  // K + 1 offsets (multiples of 4), K counts
     std::vector<uint32_t> imp;      // before level k: imp[imp_off[k] .. imp_off[k] + imp_n[k]), padded
     std::vector<int32_t> imp_off, imp_n;
     std::vector<uint32_t> imp_all;  // pairs (entry, level k) of every import, address order
+    std::vector<uint32_t> imp_run;  // imp_all with the imports of a slot pair as one entry
+    bool run_pairs = false;         // whether imp_run holds any pair
     int max_cell_n = 0, max_imp_n = 0;  // padded to multiples of 4
     // one whole region: site-updates, bytes read and written (this design)
     int64_t updates = 0, bytes_read = 0, bytes_written = 0;

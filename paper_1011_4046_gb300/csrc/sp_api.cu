@@ -55,15 +55,18 @@ struct TablesOnDevice {
 struct LatOnDevice {
     sp::LatticeTables host;
     uint32_t *d_cell = nullptr;
-    uint32_t *d_imp_all = nullptr;  // imp_all: pairs (entry, level)
+    uint32_t *d_imp_run = nullptr;  // imp_run: two words an entry
     uint64_t *d_nb = nullptr;
     int32_t *d_pcoff = nullptr;
+    uint32_t *d_wide = nullptr;  // cell_wide (null: none) and each row's slot of x = -2s
+    int32_t *d_row_x0 = nullptr;
 };
 
 // One persistent launch per region base: simulations of the same base share a
 // launch sized (shared memory, CTAs per SM) for that base alone.
 struct GroupCfg {
-    int B = 0, threads = 0, ctas_per_sm = 0, grid = 0;
+    int B = 0, threads = 0, ctas_per_sm = 0, grid = 0;  // lattice: ctas_per_sm and grid count regions
+    int groups = 1;                                     // lattice: regions per CTA
     size_t smem = 0;
 };
 
@@ -631,9 +634,11 @@ void free_plan(sp_grid *g)
     g->mbox.clear();
     for (auto &kv : g->lat) {
         cudaFree(kv.second.d_cell);
-        cudaFree(kv.second.d_imp_all);
+        cudaFree(kv.second.d_imp_run);
         cudaFree(kv.second.d_nb);
         cudaFree(kv.second.d_pcoff);
+        cudaFree(kv.second.d_wide);
+        cudaFree(kv.second.d_row_x0);
     }
     g->lat.clear();
     for (float2 *f : g->phi_odd) cudaFree(f);
@@ -890,7 +895,7 @@ int enqueue_lattice_call(sp_grid *g, const std::vector<LatLaunch> &launches, int
         const LatLaunch &l = launches[i];
         e = sp::launch_lattice_reset(l.a.ctl, l.a.Lcount, g->stream);
         if (timing && i == 0) mark(g->ev[1]);
-        if (e == cudaSuccess) e = sp::launch_lattice(l.a, l.cfg.threads, l.cfg.smem, l.cfg.grid, g->stream);
+        if (e == cudaSuccess) e = sp::launch_lattice(l.a, l.cfg.threads, l.cfg.smem, l.cfg.grid / l.cfg.groups, g->stream);
     }
     if (launches.empty() && timing) mark(g->ev[1]);
     if (timing) mark(g->ev[2]);
@@ -996,13 +1001,20 @@ int evolve_lattice(sp_grid *g, int64_t n_steps, bool trace, bool timing)
         a.n_slots = t.n_slots;
         a.n_foot = t.n_foot;
         a.Lcount = Lcount;
+        a.run_pairs = t.run_pairs;
         a.per_layer_all = (unsigned)per_layer_all;
         a.total = (unsigned)(per_layer_all * Lcount);
         a.cell = ld.d_cell;
-        a.imp_all = reinterpret_cast<const uint2 *>(ld.d_imp_all);
-        a.n_imp_all = (int)(t.imp_all.size() / 2);
+        a.imp_run = reinterpret_cast<const uint2 *>(ld.d_imp_run);
+        a.n_imp_run = (int)(t.imp_run.size() / 2);
         a.row_nb = ld.d_nb;
         a.row_pc = ld.d_pcoff;
+        a.cell_wide = reinterpret_cast<const uint2 *>(ld.d_wide);
+        a.row_x0 = ld.d_row_x0;
+        a.n_cell = (int)t.cell.size();
+        a.groups = c.groups;
+        a.bank_a = t.bank_a;
+        a.bank_b = t.bank_b;
         a.max_cell_n = t.max_cell_n;
         a.flags = g->d_lat_flags + g->lat_flag_off[gi];
         a.ctl = g->d_ctl + gi;
@@ -1171,17 +1183,26 @@ int plan_lattice(sp_grid *g, const std::vector<int> &Bs, int threads)
         if (!sp::build_lattice_tables(s, &ld.host).empty()) return SP_EINVAL;
         const sp::LatticeTables &t = ld.host;
         e = cudaMalloc((void **)&ld.d_cell, t.cell.size() * sizeof(uint32_t));
-        if (e == cudaSuccess) e = cudaMalloc((void **)&ld.d_imp_all, std::max<size_t>(t.imp_all.size(), 4) * sizeof(uint32_t));
+        if (e == cudaSuccess) e = cudaMalloc((void **)&ld.d_imp_run, std::max<size_t>(t.imp_run.size(), 4) * sizeof(uint32_t));
         if (e == cudaSuccess) e = cudaMalloc((void **)&ld.d_nb, t.row_nb.size() * sizeof(uint64_t));
         if (e == cudaSuccess) e = cudaMalloc((void **)&ld.d_pcoff, t.row_pc.size() * sizeof(int32_t));
         if (e == cudaSuccess)
             e = cudaMemcpy(ld.d_cell, t.cell.data(), t.cell.size() * sizeof(uint32_t), cudaMemcpyHostToDevice);
-        if (e == cudaSuccess && !t.imp_all.empty())
-            e = cudaMemcpy(ld.d_imp_all, t.imp_all.data(), t.imp_all.size() * sizeof(uint32_t), cudaMemcpyHostToDevice);
+        if (e == cudaSuccess && !t.imp_run.empty())
+            e = cudaMemcpy(ld.d_imp_run, t.imp_run.data(), t.imp_run.size() * sizeof(uint32_t), cudaMemcpyHostToDevice);
         if (e == cudaSuccess)
             e = cudaMemcpy(ld.d_nb, t.row_nb.data(), t.row_nb.size() * sizeof(uint64_t), cudaMemcpyHostToDevice);
         if (e == cudaSuccess)
             e = cudaMemcpy(ld.d_pcoff, t.row_pc.data(), t.row_pc.size() * sizeof(int32_t), cudaMemcpyHostToDevice);
+        if (!t.cell_wide.empty()) {
+            std::vector<int32_t> x0(t.row_xy.size());
+            for (size_t i = 0; i < x0.size(); ++i) x0[i] = sp::lat_row_base(t.row_xy[i]) - 2 * t.s;
+            if (e == cudaSuccess) e = cudaMalloc((void **)&ld.d_wide, t.cell_wide.size() * sizeof(uint32_t));
+            if (e == cudaSuccess) e = cudaMalloc((void **)&ld.d_row_x0, x0.size() * sizeof(int32_t));
+            if (e == cudaSuccess)
+                e = cudaMemcpy(ld.d_wide, t.cell_wide.data(), t.cell_wide.size() * sizeof(uint32_t), cudaMemcpyHostToDevice);
+            if (e == cudaSuccess) e = cudaMemcpy(ld.d_row_x0, x0.data(), x0.size() * sizeof(int32_t), cudaMemcpyHostToDevice);
+        }
         if (e != cudaSuccess) {
             free_plan(g);
             return SP_ENOMEM;
@@ -1192,14 +1213,17 @@ int plan_lattice(sp_grid *g, const std::vector<int> &Bs, int threads)
         const sp::LatticeTables &t = it->second.host;
         GroupCfg c;
         c.B = 4 * it->first;
-        // default (measured): 64 workers up to s = 2 (at most 76 cells a
-        // level), 128 at s = 3 and 4, 256 at s = 5, 512 at s = 6
+        // default (measured at 240^3): 64 workers up to s = 3 (1.05e11
+        // site-updates/s at s = 3, 0.80e11 with 128), 128 at s = 4 (1.384e11; 64:
+        // 0.91e11, 192: 1.21e11), 256 at s = 5, 512 at s = 6
         const int s_lat = it->first;
-        c.threads = threads ? threads : s_lat <= 2 ? 64 : s_lat <= 4 ? 128 : s_lat == 5 ? 256 : 512;
-        c.smem = sp::lattice_smem_bytes(t.n_slots, t.n_foot, t.rb_side, t.max_cell_n);
-        if (c.smem > 227 * 1024) return SP_EINVAL;
-        e = sp::lattice_occupancy(c.threads, c.smem, &c.ctas_per_sm);
-        if (e != cudaSuccess || c.ctas_per_sm < 1) return SP_EINVAL;
+        c.threads = threads ? threads : s_lat <= 3 ? 64 : s_lat <= 4 ? 128 : s_lat == 5 ? 256 : 512;
+        sp::LatConfig lc;
+        e = sp::lattice_config(t, c.threads, &lc);
+        if (e != cudaSuccess || lc.ctas_per_sm < 1) return SP_EINVAL;
+        c.smem = lc.smem;
+        c.groups = lc.groups;
+        c.ctas_per_sm = lc.ctas_per_sm * lc.groups;
         c.grid = c.ctas_per_sm * g->sm_count;
         g->groups.push_back(c);
         g->lat_flag_off.push_back(flags);

@@ -180,18 +180,23 @@ struct alignas(16) LatSimDev {
 struct LatArgs {
     const LatSimDev *sims;
     int n_sims, s, K, T;
-    int n_slots, n_foot, Lcount, pad0;
+    int n_slots, n_foot, Lcount, run_pairs;  // run_pairs: imp_run holds slot pairs
     long long fault_drop;            // region id (as in the trace) that never reports done (-1: none)
     unsigned per_layer_all, total;
     const uint32_t *cell;            // cell entries (lattice.h), all levels (16-byte aligned per level)
-    const uint2 *imp_all;            // (entry, level) of every import of a region, address order
+    const uint2 *imp_run;            // imports of a region, pairs of slots as one entry, address order
     const uint64_t *row_nb;          // (4s + 1)^2 row records: neighbour steps
     const int32_t *row_pc;           // (4s + 1)^2 row records: (pi, c) index - slot
-    int max_cell_n, n_imp_all;       // longest level's cell list (padded); imports of a region
+    int max_cell_n, n_imp_run;       // longest level's cell list (padded); entries of imp_run
     int *flags;
     Ctl *ctl;
     unsigned long long *trace;       // optional (start, end) globaltimer per region: simulation by
                                      // simulation, layer by layer (trace_base + layer * per_layer + idx)
+    // lattice_kernel: the wide entries of all levels, the slot of x = -2s per
+    // row, regions per CTA, and the row steps' residues a, b
+    const uint2 *cell_wide;
+    const int32_t *row_x0;
+    int n_cell, groups, bank_a, bank_b;
     int cell_off[4 * 6 + 1];  // per level (entries)
     int cell_n[4 * 6];
 };

@@ -42,12 +42,18 @@ int region_oct_workers();
 }  // namespace sp
 
 namespace sp {
-// The 4-cube lattice kernel (sp_lattice.cu): dynamic shared memory of one
-// region, worker counts, occupancy, the per-call reset (ticket counter,
-// error word, layer epoch) and the launch.
-size_t lattice_smem_bytes(int n_slots, int n_foot, int rb_side, int max_cell_n);
+struct LatticeTables;
+// The 4-cube lattice kernels (sp_lattice.cu): how a size runs with a worker
+// count (regions per CTA, CTAs per SM, dynamic shared memory; no CTA: it does
+// not fit), the per-call reset (ticket counter, error word, layer epoch) and
+// the launch of `grid` CTAs.
+struct LatConfig {
+    bool resident = false;  // the kernel with the whole cell list in shared memory
+    int groups = 1, ctas_per_sm = 0;
+    size_t smem = 0;
+};
 bool lattice_valid_threads(int threads);
-cudaError_t lattice_occupancy(int threads, size_t smem, int *blocks_per_sm);
+cudaError_t lattice_config(const LatticeTables &t, int threads, LatConfig *c);
 cudaError_t launch_lattice_reset(Ctl *ctl, int layers, cudaStream_t st);
 cudaError_t launch_lattice(const LatArgs &a, int threads, size_t smem, int grid, cudaStream_t st);
 }  // namespace sp
