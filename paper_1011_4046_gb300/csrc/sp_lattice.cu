@@ -183,7 +183,8 @@ __device__ __forceinline__ void load_import_batch(uint2 (&ie)[lat_imp_batch<NW>(
 template <int NW, bool PAIRS, int YS>
 __device__ __forceinline__ void issue_import_batch(const uint2 (&ie)[lat_imp_batch<NW>()], int k_lo, int k_hi, int cx,
                                                    int n0, const unsigned *s_yz, char *pcb, char *ph0, char *ph1,
-                                                   const float2 *g0, const float2 *g1, const float4 *gpc, uint32_t pair_bit)
+                                                   const float2 *g0, const float2 *g1, const float4 *gpc, uint32_t pair_bit,
+                                                   bool aligned)
 {
 #pragma unroll
     for (int u = 0; u < lat_imp_batch<NW>(); ++u) {
@@ -196,7 +197,7 @@ __device__ __forceinline__ void issue_import_batch(const uint2 (&ie)[lat_imp_bat
         const unsigned long long g = lat_site(lat_rx2s(e), yz, cx, n0);
         char *dst = (b ? ph1 : ph0) + (sl << 3);
         const float2 *src = (b ? g1 : g0) + g;
-        const bool same = ((sl ^ (int)g) & 1) == 0;  // slot and site parity
+        const bool same = aligned && ((sl ^ (int)g) & 1) == 0;  // slot and site parity, and phi on 16 bytes
         const bool both = PAIRS && (w & kLatRunPair);
         if (same && (both || (e & pair_bit)))
             cp_async16(dst - ((sl & 1) << 3), src - (g & 1));
@@ -364,11 +365,14 @@ __global__ void __launch_bounds__(lat_max_threads<NW>(), 1) lattice_kernel(const
         // levels of parity b, global parity par0 ^ b
         const float2 *const g0 = par0 ? g_odd : g_even, *const g1 = par0 ? g_even : g_odd;
         const uint32_t pair_bit = r.k_lo == 0 ? kLatImpPair : kLatImpPairRow;
+        const bool aligned = (((uintptr_t)g_even | (uintptr_t)g_odd) & 15) == 0;  // the caller's phi may not be
         for (int i0 = tid;;) {
             if (a.run_pairs)
-                issue_import_batch<NW, true, 1>(ie, r.k_lo, r.k_hi, cx, n0, s_yz, s_pcb, s_ph0, s_ph1, g0, g1, gpc, pair_bit);
+                issue_import_batch<NW, true, 1>(ie, r.k_lo, r.k_hi, cx, n0, s_yz, s_pcb, s_ph0, s_ph1, g0, g1, gpc, pair_bit,
+                                                   aligned);
             else
-                issue_import_batch<NW, false, 1>(ie, r.k_lo, r.k_hi, cx, n0, s_yz, s_pcb, s_ph0, s_ph1, g0, g1, gpc, pair_bit);
+                issue_import_batch<NW, false, 1>(ie, r.k_lo, r.k_hi, cx, n0, s_yz, s_pcb, s_ph0, s_ph1, g0, g1, gpc, pair_bit,
+                                                   aligned);
             i0 += lat_imp_batch<NW>() * NW;
             if (i0 - tid >= a.n_imp_run) break;
             load_import_batch<NW>(ie, a.imp_run, a.n_imp_run, i0);
@@ -562,10 +566,13 @@ __global__ void __launch_bounds__(NW, lat_min_blocks<NW>())
         for (int i0 = tid;;) {
             const float2 *const g0 = par0 ? g_odd : g_even, *const g1 = par0 ? g_even : g_odd;
             const uint32_t pair_bit = r.k_lo == 0 ? kLatImpPair : kLatImpPairRow;
+            const bool aligned = (((uintptr_t)g_even | (uintptr_t)g_odd) & 15) == 0;  // the caller's phi may not be
             if (a.run_pairs)
-                issue_import_batch<NW, true, 4>(ie, r.k_lo, r.k_hi, cx, n0, &s_row->yz, s_pcb, s_ph0, s_ph1, g0, g1, gpc, pair_bit);
+                issue_import_batch<NW, true, 4>(ie, r.k_lo, r.k_hi, cx, n0, &s_row->yz, s_pcb, s_ph0, s_ph1, g0, g1, gpc, pair_bit,
+                                                   aligned);
             else
-                issue_import_batch<NW, false, 4>(ie, r.k_lo, r.k_hi, cx, n0, &s_row->yz, s_pcb, s_ph0, s_ph1, g0, g1, gpc, pair_bit);
+                issue_import_batch<NW, false, 4>(ie, r.k_lo, r.k_hi, cx, n0, &s_row->yz, s_pcb, s_ph0, s_ph1, g0, g1, gpc, pair_bit,
+                                                   aligned);
             i0 += lat_imp_batch<NW>() * NW;
             if (i0 >= a.n_imp_run) break;
             load_import_batch<NW>(ie, a.imp_run, a.n_imp_run, i0);
