@@ -8,8 +8,9 @@
  * through final surfaces, so each region can be evolved on its own as soon as
  * its predecessors are done, and a manager hands ready regions to workers
  * (Sec. 4).  Here a region is a pyramid, inverted pyramid or wedge of B^3
- * lattice cells and B/2 leapfrog steps; the manager is a device work queue
- * and the workers are the CTAs of one persistent kernel.  The model equation,
+ * lattice cells and B/2 leapfrog steps; the managers are warps that take
+ * regions from a common order and wait for their predecessors, the workers the
+ * other threads of one persistent kernel.  The model equation,
  * in conformal time tau with a = (tau / tau_ref)^nu, is
  *
  *   phi'' + 2 (nu / tau) phi' - Lap7 phi + a^2 lambda (|phi|^2 - eta^2) phi = 0,
@@ -56,7 +57,7 @@ extern "C" {
 
 /* ---- flags of sp_evolve ---- */
 #define SP_ASYNC 1u      /* return without synchronising the stream */
-#define SP_MONOLITHIC 2u /* whole-grid sweep, one launch per step (comparator) */
+#define SP_MONOLITHIC 2u /* whole-grid sweep, a launch per step or per two steps (comparator) */
 #define SP_RESTART 4u    /* treat the current state as level 0 (tau = tau0) */
 #define SP_TRACE 8u      /* record (start, end) globaltimer ns of every region (SP_SURF_TRACE) */
 #define SP_TIMING 16u    /* record CUDA events around each launch of the call (SP_SURF_TIMING) */
@@ -68,7 +69,7 @@ extern "C" {
 #define SP_SURF_TRACE 2   /* per-region (start, end) ns of the last region launch */
 #define SP_SURF_WINDING 3 /* int8 plaquette windings [3][sites] */
 #define SP_SURF_PLAN 4    /* one sp_plan_info */
-#define SP_SURF_TIMING 5  /* double[3]: ms of the queue reset, the region kernel and the
+#define SP_SURF_TIMING 5  /* double[3]: ms of the order's reset, the region kernel and the
                              remainder sweep of the last SP_TIMING call (events on the stream) */
 #define SP_SURF_LEVEL 7    /* int64 (host memory): the simulation's current level n; readable and
                               writable -- a checkpoint is SP_SURF_STATE plus SP_SURF_LEVEL */
@@ -154,7 +155,8 @@ typedef struct {
 } sp_diag;
 
 /* Plan summary of one simulation (traffic is of this design, per band;
- * threads, ctas_per_sm and grid are those of the launch of its base). */
+ * threads, ctas_per_sm and grid are those of the launch of its base: workers
+ * per region, regions resident per SM and in all; base 32 counts CTAs). */
 typedef struct {
     int32_t base_B, threads, ctas_per_sm, grid;
     int64_t regions_per_band;
@@ -205,21 +207,22 @@ int sp_grid_create(const sp_params *p, int32_t n_sims, void *const *state_dev, v
  *                (4, 8, 12, 16, 20 or 24; 4s levels per region); every n[d]
  *                a multiple of B; 0 takes 16 where it divides, else 8, else
  *                4; SP_AUTOTUNE times the sizes that divide every side.
- *   block_shape: worker threads per CTA (64, 128, 256, 320, 384, 480, 512 or 768;
+ *   block_shape: worker threads per region (64, 128, 256, 320, 384, 480, 512 or 768;
  *                lattice plans: 64, 128, 192, 256 or 512 per region
  *                and no manager warp (default: 64 up to s = 3, 128 at s = 4, 256 at
  *                s = 5, 512 at s = 6);
  *                every worker taking every step of a region); one manager
  *                warp is added.  0 for the default of each base (64 for
- *                bases 4 and 8, 384 for 16); SP_AUTOTUNE to time the
- *                candidates for the largest base (64, 128 for base 8; 320,
+ *                base 4; 384 for 16; for 8, by the regions of a type on an SM,
+ *                64; 128 up to five, 256 up to a half); SP_AUTOTUNE to time the
+ *                candidates for the largest base (64, 128, 256 for base 8; 320,
  *                384, 480 for base 16), smaller bases keeping their default.
  *                A value applies to every base.
  *                The autotuner runs 16-step calls on scratch copies of the
  *                current state (sides above 128 cells are cut to 128 or 120),
  *                on the grid's stream; the state itself is not modified.
- *   order      : SP_ORDER_STATIC (ready regions are popped in the order they
- *                became ready) or SP_ORDER_LEARNED (each call predicts every
+ *   order      : SP_ORDER_STATIC (regions are taken in a fixed order of bands,
+ *                phases and positions; base 32: as they became ready) or SP_ORDER_LEARNED (each call predicts every
  *                region's cost from its features with the model at
  *                model_path and pops the predicted-expensive quarter first,
  *                then the next quarter, ...).  The order never changes results.
@@ -232,8 +235,9 @@ int sp_region_plan(sp_grid *g, int32_t base_B, int32_t block_shape, int32_t orde
  * sp_evolve -- advance every simulation by n_steps leapfrog steps.
  * Paper Sec. 4: a manager holds the pool of regions whose predecessors are
  * done and hands one to each worker that reports its previous region
- * finished; here the pool is a device work queue and the workers are the
- * CTAs of one persistent launch per region base.
+ * finished; here managers and workers are warps of one persistent launch per
+ * region base, and the pool is a fixed order from which each manager takes the
+ * next region (learned order and base 32: a device work queue).
  * Whole bands of B/2 steps run as regions in one persistent launch per
  * distinct base (largest base first, each launch sized for its base); a
  * remainder of fewer than B/2 steps runs as whole-grid steps with the same

@@ -49,6 +49,7 @@ struct TablesOnDevice {
     unsigned short *d_imp = nullptr;
     int2 *d_exp = nullptr;
     sp::Succ *d_reuse = nullptr;  // mailbox-reuse successors, kMaxSameSucc per type
+    sp::Pred *d_preds = nullptr;  // predecessors by band parity and type, kMaxPreds each
 };
 
 // The 4-cube lattice tables of one size s (lattice.h) on the device.
@@ -65,8 +66,8 @@ struct LatOnDevice {
 // One persistent launch per region base: simulations of the same base share a
 // launch sized (shared memory, CTAs per SM) for that base alone.
 struct GroupCfg {
-    int B = 0, threads = 0, ctas_per_sm = 0, grid = 0;  // lattice: ctas_per_sm and grid count regions
-    int groups = 1;                                     // lattice: regions per CTA
+    int B = 0, threads = 0, ctas_per_sm = 0, grid = 0;  // ctas_per_sm and grid count resident regions (base 32: CTAs)
+    int groups = 1;                                     // regions per CTA
     size_t smem = 0;
 };
 
@@ -211,6 +212,8 @@ struct sp_grid {
     // launch scratch
     int *d_counters = nullptr, *d_queue = nullptr;
     size_t cap_counters = 0, cap_queue = 0;
+    int *d_flags = nullptr;  // ticket order: the launch epoch, then a done flag per region
+    size_t cap_flags = 0;
     sp::Ctl *d_ctl = nullptr;
     sp::SimDev *d_sims = nullptr;
     size_t cap_sims = 0;
@@ -335,6 +338,50 @@ int upload_reuse(const sp::TileTables &t, sp::Succ **d_reuse)
     if (cudaMalloc((void **)d_reuse, reuse.size() * sizeof(sp::Succ)) != cudaSuccess) return SP_ENOMEM;
     if (cudaMemcpy(*d_reuse, reuse.data(), reuse.size() * sizeof(sp::Succ), cudaMemcpyHostToDevice) != cudaSuccess)
         return SP_ECUDA;
+    return SP_OK;
+}
+
+// The predecessors of every type by parity of its band (the inverse of the
+// successor patterns), for the ticket order: the same band's, the previous
+// band's, those of mailbox reuse.  Checks what that order relies on: a
+// same-band predecessor's type is of an earlier phase, and the counts are the
+// planner's.
+int build_preds(const sp::TileTables &t, sp::TablesDev *h, std::vector<sp::Pred> *preds)
+{
+    preds->assign((size_t)2 * sp::kTypes * sp::kMaxPreds, sp::Pred{{0, 0, 0}, 0});
+    for (int q = 0; q < 2; ++q)
+        for (int S = 0; S < sp::kTypes; ++S) {
+            sp::Pred *out = preds->data() + (size_t)(q * sp::kTypes + S) * sp::kMaxPreds;
+            int n = 0;
+            bool ok = true;
+            auto add = [&](int type, int prev, const sp::Succ &e) {
+                if (n >= sp::kMaxPreds) {
+                    ok = false;
+                    return;
+                }
+                out[n].type_prev = (unsigned char)(type | prev << 3);
+                for (int d = 0; d < 3; ++d) out[n].e[d] = (signed char)-e.e[d];
+                ++n;
+            };
+            for (int from = 0; from < sp::kTypes; ++from)
+                for (const sp::Succ &e : t.same_succ[from])
+                    if (e.type == S) {
+                        ok = ok && __builtin_popcount((unsigned)from) < __builtin_popcount((unsigned)S);
+                        add(from, 0, e);
+                    }
+            ok = ok && n == t.same_preds[S];
+            h->pred_n[S][0] = (unsigned char)n;
+            for (const sp::Succ &e : t.next_succ[q])
+                if (e.type == S) add(sp::kTypes - 1, 1, e);
+            ok = ok && n == t.same_preds[S] + t.prev_preds[S];
+            h->pred_n[S][1] = (unsigned char)n;
+            for (int from = 0; from < sp::kTypes; ++from)
+                for (const sp::Succ &e : t.reuse_succ[from])
+                    if (e.type == S) add(from, 1, e);
+            ok = ok && n == t.same_preds[S] + t.prev_preds[S] + t.reuse_preds[S];
+            h->pred_n[S][2] = (unsigned char)n;
+            if (!ok) return SP_EINVAL;
+        }
     return SP_OK;
 }
 
@@ -588,10 +635,15 @@ int build_device_tables(sp_grid *g, int B)
     up((void **)&td.d_imp, imp.data(), imp.size() * sizeof(unsigned short));
     up((void **)&td.d_exp, ex.data(), ex.size() * sizeof(int2));
     up((void **)&td.d_reuse, reuse.data(), reuse.size() * sizeof(sp::Succ));
+    std::vector<sp::Pred> preds;
+    if (build_preds(t, &h, &preds) != SP_OK) return SP_EINVAL;
+    up((void **)&td.d_preds, preds.data(), preds.size() * sizeof(sp::Pred));
     h.imp = td.d_imp;
     h.exp = td.d_exp;
     h.reuse = td.d_reuse;
+    h.preds = td.d_preds;
     if (e != cudaSuccess) {
+        cudaFree(td.d_preds);
         cudaFree(td.d_imp);
         cudaFree(td.d_exp);
         cudaFree(td.d_reuse);
@@ -622,6 +674,7 @@ void free_plan(sp_grid *g)
         cudaFree(kv.second.d_imp);
         cudaFree(kv.second.d_exp);
         cudaFree(kv.second.d_reuse);
+        cudaFree(kv.second.d_preds);
         cudaFree(kv.second.d_dev);
         cudaFree(kv.second.d_oimp);
         cudaFree(kv.second.d_oexp);
@@ -666,7 +719,24 @@ int choose_B(const sp_params &p, int requested)
     return -1;
 }
 
-int default_threads(int B) { return B <= 8 ? 64 : B == 32 ? sp::region_oct_workers() : 384; }
+// Default workers of a base-8 region.  Many regions: 64, of which eight fit an
+// SM.  Where the widest phase (three region types) leaves an SM few regions at
+// a time, the chain of phases counts, and more workers shorten each region
+// (one simulation, 64 steps, us with 64 / 128 / 256 workers: 24^3 - / 431 / 401,
+// 32^3 564 / 432 / 433, 40^3 570 / 489 / 511, 48^3 654 / 535, 64^3 734 / 675,
+// 72^3 827 / 798, 80^3 934 / 985, 96^3 1255 / 1535).
+int base8_threads(long long tiles, int sms) { return 2 * tiles <= sms ? 256 : tiles <= 5ll * sms ? 128 : 64; }
+
+// Default workers of a region of base B in a plan with the bases Bs.
+int default_threads(const sp_grid *g, const std::vector<int> &Bs, int B)
+{
+    if (B == 32) return sp::region_oct_workers();
+    if (B != 8) return B < 8 ? 64 : 384;
+    long long tiles = 0;  // regions of a type, of all simulations of this base
+    for (int s = 0; s < g->n_sims; ++s)
+        if (Bs[s] == B) tiles += (long long)(g->p[s].n[0] / B) * (g->p[s].n[1] / B) * (g->p[s].n[2] / B);
+    return base8_threads(tiles, g->sm_count);
+}
 
 // Pending device error of the last region launch -> SP code.
 int collect_device_error(sp_grid *g)
@@ -804,7 +874,8 @@ int enqueue_region_call(sp_grid *g, const std::vector<GroupLaunch> &groups, int6
         if (timing && gi == 0) mark(g->ev[1]);
         if (e == cudaSuccess)
             e = gl.cfg.B == 32 ? sp::launch_region_oct(a, gl.cfg.smem, gl.cfg.grid / 8, g->stream)
-                               : sp::launch_region(a, gl.cfg.threads, gl.cfg.B, gl.cfg.smem, gl.cfg.grid, g->stream);
+                               : sp::launch_region(a, gl.cfg.threads, gl.cfg.B, gl.cfg.groups, gl.cfg.smem,
+                                                   gl.cfg.grid / gl.cfg.groups, g->stream);
     }
     if (groups.empty() && timing) mark(g->ev[1]);
     if (timing) mark(g->ev[2]);
@@ -1105,13 +1176,13 @@ int plan_fixed(sp_grid *g, const std::vector<int> &Bs, int threads, int order, c
             continue;
         }
         const bool mine = threads && (!largest_only || c.B == g->max_B);
-        c.threads = mine ? threads : default_threads(c.B);
-        int n_in = 0;
-        for (int s = 0; s < g->n_sims; ++s) n_in += g->B[s] == c.B;
-        c.smem = sp::region_smem_bytes(c.B, 1, n_in, it->second.dev.imp_n);
-        if (c.smem > 227 * 1024) return SP_EINVAL;
-        e = sp::region_occupancy(c.threads, c.B, c.smem, &c.ctas_per_sm);
-        if (e != cudaSuccess || c.ctas_per_sm < 1) return SP_EINVAL;
+        c.threads = mine ? threads : default_threads(g, g->B, c.B);
+        sp::RegionConfig rc;
+        e = sp::region_config(c.threads, c.B, it->second.dev.imp_n, &rc);
+        if (e != cudaSuccess || rc.ctas_per_sm < 1) return SP_EINVAL;
+        c.smem = rc.smem;
+        c.groups = rc.groups;
+        c.ctas_per_sm = rc.ctas_per_sm * rc.groups;
         c.grid = c.ctas_per_sm * g->sm_count;
         g->groups.push_back(c);
     }
@@ -1318,9 +1389,9 @@ int autotune(sp_grid *g, int base_B, int block_shape, std::vector<int> *best_B, 
         const int maxB = *std::max_element(Bs.begin(), Bs.end());
         std::vector<int> shapes;
         if (block_shape != SP_AUTOTUNE)
-            shapes.push_back(block_shape ? block_shape : default_threads(maxB));
+            shapes.push_back(block_shape ? block_shape : default_threads(t, Bs, maxB));
         else if (maxB <= 8)
-            shapes = {64, 128};
+            shapes = {64, 128, 256};
         else
             shapes = {320, 384, 480};
         for (int nt : shapes) {
@@ -1338,7 +1409,7 @@ int autotune(sp_grid *g, int base_B, int block_shape, std::vector<int> *best_B, 
                 return rc;
             }
             ++g->tune.candidates;
-            const bool is_default = Bs == policies.back() && nt == default_threads(maxB);
+            const bool is_default = Bs == policies.back() && nt == default_threads(t, Bs, maxB);
             if (is_default) g->tune.default_ms = ms;
             if (!have || ms < best) {
                 best = ms;
@@ -1623,7 +1694,7 @@ int sp_evolve(sp_grid *g, int64_t n_steps, uint32_t flags)
         std::vector<sp::SimDev> sims;
         std::vector<int> sim_of;
         std::vector<GroupLaunch> launches;
-        unsigned all_total = 0, max_total = 0;
+        unsigned all_total = 0, max_total = 0, max_flags = 0;  // max_total: of the launches with a ready queue
         g->last_tile_base.assign(g->n_sims, 0);
         g->last_tiles.assign(g->n_sims, 0);
         const bool learned = g->order == SP_ORDER_LEARNED && g->model;
@@ -1638,6 +1709,7 @@ int sp_evolve(sp_grid *g, int64_t n_steps, uint32_t flags)
             gl.sim_off = sims.size();
             gl.roff = all_total;
             unsigned total = 0, seeds = 0;
+            int tiles_in = 0;
             for (int s = 0; s < g->n_sims; ++s) {
                 if (g->B[s] != B) continue;
                 sp::SimDev d;
@@ -1656,6 +1728,7 @@ int sp_evolve(sp_grid *g, int64_t n_steps, uint32_t flags)
                 d.tile_base = total;
                 d.tiles = (unsigned)tiles;
                 d.seed_base = seeds;
+                d.tile_first = tiles_in;
                 d.coef = g->d_coef + (size_t)s * n_steps;
                 d.q = phys_const(g->p[s]);
                 d.phi = g->phi[s];
@@ -1671,6 +1744,7 @@ int sp_evolve(sp_grid *g, int64_t n_steps, uint32_t flags)
                 g->last_tiles[s] = d.tiles;
                 total += d.tiles;
                 seeds += (unsigned)d.Jtot * (unsigned)g->tables[B].seed_types;
+                tiles_in += d.Jtot;
                 sims.push_back(d);
                 sim_of.push_back(s);
             }
@@ -1682,17 +1756,25 @@ int sp_evolve(sp_grid *g, int64_t n_steps, uint32_t flags)
             ra.n_sims = (int)(sims.size() - gl.sim_off);
             ra.total = total;
             ra.n_seed = seeds;
+            ra.all_tiles = tiles_in;
             ra.ctl = g->d_ctl + launches.size();
             const long long fd = (long long)g->fault_drop - (long long)all_total;
             ra.fault_drop = (g->fault_drop >= 0 && fd >= 0 && fd < (long long)total) ? (int)fd : -1;
             launches.push_back(gl);
             all_total += total;
-            max_total = std::max(max_total, total);
+            if (learned || B == 32)
+                max_total = std::max(max_total, total);
+            else
+                max_flags = std::max(max_flags, total);
         }
         if (!launches.empty()) {
             e = grow(&g->d_sims, &g->cap_sims, sims.size());
             if (e == cudaSuccess) e = grow(&g->d_counters, &g->cap_counters, max_total);
             if (e == cudaSuccess) e = grow(&g->d_queue, &g->cap_queue, max_total);
+            if (e == cudaSuccess && max_flags && g->cap_flags < (size_t)max_flags + 1) {
+                e = grow(&g->d_flags, &g->cap_flags, (size_t)max_flags + 1);
+                if (e == cudaSuccess) e = cudaMemsetAsync(g->d_flags, 0, g->cap_flags * sizeof(int), g->stream);
+            }
             if (e == cudaSuccess && trace) e = grow(&g->d_trace, &g->cap_trace, 2 * (size_t)all_total);
             if (e == cudaSuccess && feats) e = grow(&g->d_feat, &g->cap_feat, (size_t)SP_MODEL_FEATURES * all_total);
             if (e == cudaSuccess && feats) e = grow(&g->d_simf, &g->cap_simf, sims.size());
@@ -1702,6 +1784,10 @@ int sp_evolve(sp_grid *g, int64_t n_steps, uint32_t flags)
                 gl.a.sims = g->d_sims + gl.sim_off;
                 gl.a.counters = g->d_counters;
                 gl.a.queue = g->d_queue;
+                if (!learned && gl.cfg.B != 32) {
+                    gl.a.epoch = g->d_flags;
+                    gl.a.flags = g->d_flags + 1;
+                }
                 gl.a.trace = trace ? g->d_trace + 2 * (size_t)gl.roff : nullptr;
                 gl.a.prio = learned ? g->d_prio + gl.roff : nullptr;
             }
@@ -2012,6 +2098,7 @@ int sp_destroy(sp_grid *g)
     }
     cudaFree(g->d_counters);
     cudaFree(g->d_queue);
+    cudaFree(g->d_flags);
     cudaFree(g->d_ctl);
     cudaFree(g->d_sims);
     cudaFree(g->d_coef);

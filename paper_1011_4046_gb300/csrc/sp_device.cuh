@@ -39,6 +39,14 @@ struct alignas(16) TypeMeta {
     int n_reuse, reuse_preds;
 };
 
+// A predecessor of a region: the region of this type one band earlier (prev)
+// or in the same band, at the position offset e.
+struct Pred {
+    signed char e[3];
+    unsigned char type_prev;  // type | prev << 3
+};
+constexpr int kMaxPreds = 64;  // per type: two per lane of the manager warp
+
 // Geometry and surface-routing tables for one base size, in device memory.
 //
 // Import lists are 16-bit: a full-state import holds the cell's (pi, c) index
@@ -62,6 +70,12 @@ struct alignas(16) TablesDev {
     const Succ *reuse;
     const unsigned short *imp;  // all import lists, global memory
     const int2 *exp;            // all export entries, global memory
+    // predecessors by parity of the region's band and type, kMaxPreds each,
+    // global memory: the same band's, the previous band's, then those whose
+    // mailbox the region writes; pred_n counts the first one, two, three kinds
+    const Pred *preds;
+    unsigned char pred_n[kTypes][3];
+    unsigned char pad_pred[24 - 3 * kTypes + 16];
 };
 
 // Levels per band of the octant (cluster) kernel: bases up to 32.
@@ -132,7 +146,8 @@ struct alignas(16) SimDev {
     // base 32: the octant tables of the cluster kernel (the dependency
     // pattern stays in tab); nullptr otherwise
     const TablesOct *oct;
-    long long pad_oct;
+    int tile_first;  // positions of the launch's earlier simulations (ticket order)
+    int pad_oct;
 };
 
 // Priority buckets of the learned ordering (bucket 0 is queued first).
@@ -219,7 +234,13 @@ struct RegionArgs {
     // Host-injected failure (failure-detection tests): the region with this
     // launch id finishes but never releases its successors; -1 = none.
     int fault_drop;
-    int pad_;
+    // Ticket order (static order, bases up to 16): regions are handed out in
+    // the order of their bands and, within a band, of their types' phases,
+    // positions running over all simulations (all_tiles in all); flags[region
+    // id] holds the epoch of the last launch in which the region finished.
+    int all_tiles;
+    int *flags;   // nullptr: ready queue
+    int *epoch;   // of this launch, set by its reset
 };
 
 static_assert(sizeof(TablesDev) % 16 == 0, "tables are copied in 16-byte units");

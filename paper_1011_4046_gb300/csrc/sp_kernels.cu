@@ -74,6 +74,16 @@ __global__ void reset_kernel(RegionArgs a)
     a.queue[t] = (t < a.n_seed && !a.prio) ? seed_region(a, t) : -1;
 }
 
+// Ticket order: a fresh ticket counter and error word, and an epoch above every
+// done flag written before.
+__global__ void ticket_reset_kernel(Ctl *ctl, int *epoch)
+{
+    ctl->head = 0;
+    ctl->error = 0;
+    ctl->error_info = 0;
+    ++*epoch;
+}
+
 // Learned ordering: seeds per bucket (after reset_kernel zeroed the counts).
 __global__ void seed_count_kernel(RegionArgs a)
 {
@@ -128,8 +138,6 @@ __global__ void seed_kernel(RegionArgs a)
 // level-(k-1) buffer and from (pi, c) of cells outside A(k) (the planner checks
 // this), while level k writes the other buffer and (pi, c) of A(k).  Their
 // table entries are loaded into registers before the compute.
-constexpr int kWorkerBarrier = 1;
-
 static_assert(sizeof(SimDev) / 16 <= 32, "the manager warp copies a descriptor with one int4 per lane");
 
 // Export entries of a level are loaded into registers before the compute of
@@ -146,7 +154,26 @@ constexpr int kExportBatch = 4;
 // throughput grows almost linearly with the regions it holds); 256 and more
 // serve base 16, one CTA per SM.
 __host__ __device__ constexpr int region_cells_per_step(int nw) { return nw <= 128 ? 1 : 2; }
-__host__ __device__ constexpr int region_min_blocks(int nw) { return nw <= 64 ? 6 : nw <= 128 ? 4 : 1; }
+// Most threads of a CTA (workers and manager warps of its groups), which set the
+// register budget: eight regions of 64 workers, four of 128, one of more.
+__host__ __device__ constexpr int region_max_groups(int nw) { return nw <= 64 ? 8 : nw <= 128 ? 4 : 1; }
+__host__ __device__ constexpr int region_max_threads(int nw) { return region_max_groups(nw) * (nw + 32); }
+
+// What one of several groups shares beside its buffers: descriptor and decoded
+// region of each handoff slot, mailbox base by consumer code (type | offset bits
+// << 3), and the handoff with its manager.
+struct alignas(16) GroupShared {
+    SimDev sd[2];
+    RegionInfo ri[2];
+    float2 *mb[64];
+    int slot[2], handoff, done, abort;
+};
+
+__host__ __device__ constexpr size_t region_group_bytes(int B)
+{
+    return (size_t)2 * (B + 2) * (B + 2) * (B + 2) * sizeof(float2) + (size_t)B * B * B * sizeof(float4) +
+           kMaxHDev * sizeof(LevelCoef);
+}
 
 __device__ __forceinline__ void export_one(int2 e, float2 *const *mb_of, const float2 *__restrict__ phi,
                                            const float4 *__restrict__ pc)
@@ -210,15 +237,30 @@ __device__ __forceinline__ void import_level(const float2 *__restrict__ mb, int 
 // block: a block pair along z spans all sixteen 8-byte bank pairs of a phi
 // buffer (pitch B+2 = 2 mod 16 cells, plane pitch = 4 mod 16), and pc_slot
 // gives the block's eight (pi, c) pairs eight different bank groups.
-__device__ __forceinline__ void block_cell(int j, const Box3 &A, int a, int c, float rc, float ra, int &ux, int &uy,
-                                           int &uz)
+struct LevelBox {
+    Box3 A;
+    float rc, ra;
+    int a, c, cnt;
+    __device__ __forceinline__ void load(const TypeMeta &M, int k)
+    {
+        A = M.active[k];
+        rc = M.rcp_active[k][0];
+        ra = M.rcp_active[k][1];
+        const int w0 = A.hi[0] - A.lo[0], w2 = A.hi[2] - A.lo[2];
+        cnt = w0 * (A.hi[1] - A.lo[1]) * w2;
+        a = w0 >> 1;
+        c = w2 >> 1;
+    }
+};
+
+__device__ __forceinline__ void block_cell(int j, const LevelBox &L, int &ux, int &uy, int &uz)
 {
     const int m = j >> 3;
-    const int r = fdiv(m, rc);   // m / c
-    const int jj = fdiv(r, ra);  // r / a
-    ux = A.lo[0] + 2 * (r - jj * a) + (j & 1);
-    uy = A.lo[1] + 2 * jj + ((j >> 1) & 1);
-    uz = A.lo[2] + 2 * (m - r * c) + ((j >> 2) & 1);
+    const int r = fdiv(m, L.rc);   // m / c
+    const int jj = fdiv(r, L.ra);  // r / a
+    ux = L.A.lo[0] + 2 * (r - jj * L.a) + (j & 1);
+    uy = L.A.lo[1] + 2 * jj + ((j >> 1) & 1);
+    uz = L.A.lo[2] + 2 * (m - r * L.c) + ((j >> 2) & 1);
 }
 
 // Shared-memory slot of the (pi, c) pair of the cell at local u-coordinates.
@@ -228,43 +270,31 @@ __device__ __forceinline__ int pc_slot_of(int ux, int uy, int uz, int B)
     return (z * B + y) * B + (x ^ ((((y & 1) << 1) | ((z & 1) << 2)) & (B - 1)));
 }
 
-// One site of level k (linear index i, see block_cell).
-__device__ __forceinline__ void evolve_cell(int i, const Box3 &A, int a, int c, float rc, float ra, int P, int PP,
-                                            int B, const float2 *__restrict__ prev_buf, float2 *__restrict__ cur,
-                                            float4 *__restrict__ pc_s, const LevelCoef &co, const PhysConst &q)
-{
-    int ux, uy, uz;
-    block_cell(i, A, a, c, rc, ra, ux, uy, uz);
-    const int pidx = (uz * P + uy) * P + ux;
-    const int cidx = pc_slot_of(ux, uy, uz, B);
-    const float4 pc = pc_s[cidx];
-    float2 pi = make_float2(pc.x, pc.y), cc = make_float2(pc.z, pc.w);
-    const float2 nphi = site_update(prev_buf[pidx], prev_buf[pidx - 1], prev_buf[pidx + 1], prev_buf[pidx - P],
-                                    prev_buf[pidx + P], prev_buf[pidx - PP], prev_buf[pidx + PP], pi, cc, co, q);
-    cur[pidx] = nphi;
-    pc_s[cidx] = make_float4(pi.x, pi.y, cc.x, cc.y);
-}
-
-// U cells of level k, linear indices i, i + stride, ... (all < cnt): every
-// input is loaded before any result is stored, so the U updates are
-// independent instruction streams (the compiler cannot prove that a store to
-// one cell's (pi, c) does not alias another cell's load).
+// Buffer and (pi, c) indices of U cells of level k, linear indices i, i +
+// stride, ... (see block_cell); past the end of the level they are unused.
 template <int U>
-__device__ __forceinline__ void evolve_cells(int i, int stride, const Box3 &A, int a, int cz, float rc, float ra,
-                                             int P, int PP, int B, const float2 *__restrict__ prev_buf,
-                                             float2 *__restrict__ cur, float4 *__restrict__ pc_s, const LevelCoef &co,
-                                             const PhysConst &q)
+__device__ __forceinline__ void cell_indices(int i, int stride, const LevelBox &L, int P, int B, int (&pidx)[U],
+                                             int (&cidx)[U])
 {
-    int pidx[U], cidx[U];
-    float2 c[U], xm[U], xp[U], ym[U], yp[U], zm[U], zp[U];
-    float4 pc[U];
 #pragma unroll
     for (int u = 0; u < U; ++u) {
         int ux, uy, uz;
-        block_cell(i + u * stride, A, a, cz, rc, ra, ux, uy, uz);
+        block_cell(i + u * stride, L, ux, uy, uz);
         pidx[u] = (uz * P + uy) * P + ux;
         cidx[u] = pc_slot_of(ux, uy, uz, B);
     }
+}
+
+// U cells of level k: every input is loaded before any result is stored, so
+// the U updates are independent instruction streams (the compiler cannot prove
+// that a store to one cell's (pi, c) does not alias another cell's load).
+template <int U>
+__device__ __forceinline__ void evolve_cells(const int (&pidx)[U], const int (&cidx)[U], int P, int PP,
+                                             const float2 *__restrict__ prev_buf, float2 *__restrict__ cur,
+                                             float4 *__restrict__ pc_s, const LevelCoef &co, const PhysConst &q)
+{
+    float2 c[U], xm[U], xp[U], ym[U], yp[U], zm[U], zp[U];
+    float4 pc[U];
 #pragma unroll
     for (int u = 0; u < U; ++u) {
         const int p = pidx[u];
@@ -423,52 +453,245 @@ __device__ void manager_loop(const RegionArgs &a, const TablesDev *s_tabs, int *
     }
 }
 
+constexpr unsigned kPhaseOrder = 0x76534210u;  // the region types by number of inverted axes
+
+// The region of ticket t: bands in order, within a band the types by phase (a
+// predecessor's type is a subset of the region's, one phase or more earlier),
+// within a type the positions of all simulations.  Region ids stay those of
+// the queue (simulation by simulation).
+__device__ __forceinline__ RegionInfo decode_ticket(const RegionArgs &a, unsigned t, int *id)
+{
+    RegionInfo r;
+    const unsigned all = (unsigned)a.all_tiles;
+    const unsigned run = t / all, pos = t - run * all;
+    r.band = (int)(run >> 3);
+    r.S = (int)(kPhaseOrder >> (4 * (run & 7u))) & 7;
+    int lo = 0, hi = a.n_sims - 1;
+    while (lo < hi) {
+        const int mid = (lo + hi + 1) >> 1;
+        if ((unsigned)a.sims[mid].tile_first <= pos)
+            lo = mid;
+        else
+            hi = mid - 1;
+    }
+    const SimDev &sd = a.sims[lo];
+    r.sim = lo;
+    r.jl = (int)(pos - (unsigned)sd.tile_first);
+    r.j[0] = r.jl % sd.J[0];
+    r.j[1] = (r.jl / sd.J[0]) % sd.J[1];
+    r.j[2] = r.jl / (sd.J[0] * sd.J[1]);
+    *id = (int)(sd.tile_base + (unsigned)((r.band * 8 + r.S) * sd.Jtot + r.jl));
+    return r;
+}
+
+// Flag of predecessor i of region r, or nullptr when it has fewer.
+__device__ __forceinline__ const int *pred_flag(const RegionArgs &a, const SimDev &sd, const TablesDev &T, const RegionInfo &r,
+                                                int i)
+{
+    const int kinds = r.band == 0 ? 0 : sd.mb_reuse ? 2 : 1;
+    if (i >= T.pred_n[r.S][kinds]) return nullptr;
+    const Pred p = T.preds[((r.band & 1) * kTypes + r.S) * kMaxPreds + i];
+    int jc = 0, mul = 1;
+    for (int d = 0; d < 3; ++d) {
+        int v = r.j[d] + p.e[d];
+        v += (v < 0) ? sd.J[d] : 0;
+        v -= (v >= sd.J[d]) ? sd.J[d] : 0;
+        jc += v * mul;
+        mul *= sd.J[d];
+    }
+    const int band = r.band - (p.type_prev >> 3);
+    return a.flags + (sd.tile_base + (unsigned)((band * 8 + (p.type_prev & 7)) * sd.Jtot + jc));
+}
+
+// Manager warp in ticket order: takes the next ticket, stages its region while
+// the worker evolves the current one, polls the done flags of the region's
+// predecessors (two per lane), hands it over, and reports the finished region
+// by its own flag.  No queue and no counters: a release is one fence and one
+// store where decrementing every successor and pushing the ready ones took
+// about 3 us, as long as a base-8 region, and all managers shared the queue's
+// head and tail.  Tickets are taken in a topological order and every ticket is
+// held by a resident manager whose worker has only smaller ones before it,
+// so the waits end; each is bounded anyway.
+__device__ void manager_tickets(const RegionArgs &a, const TablesDev *s_tabs, int *s_slot, SimDev *s_sd, RegionInfo *s_ri,
+                                int *s_handoff, int *s_done, bool prefetch)
+{
+    const int lane = threadIdx.x & 31;
+    const unsigned long long limit = a.ctl->wait_limit_ns;
+    const int epoch = *(volatile int *)a.epoch;
+    int seq = 0;       // handoffs made
+    int pending = -1;  // region handed at seq, not yet reported
+    unsigned t = 0;
+    if (lane == 0) t = atomicAdd(&a.ctl->head, 1u);
+    t = __shfl_sync(0xffffffffu, t, 0);
+    int next = -1;     // region of ticket t, staged; -1: no more, -2: stop
+    bool staged = false, ready = false;
+    const int *f0 = nullptr, *f1 = nullptr;
+    unsigned long long t0 = globaltimer_ns(), t_progress = t0;
+    auto report = [&]() {
+        if (lane == 0 && pending != a.fault_drop) {
+            fence_acq_rel_gpu();  // the worker's surfaces (its done flag was acquired) before the region's flag
+            st_relaxed_gpu(a.flags + pending, epoch);
+        }
+        pending = -1;
+    };
+    for (unsigned spin = 0;; ++spin) {
+        if (!staged) {
+            staged = true;
+            ready = t >= a.total;
+            next = -1;
+            if (!ready) {
+                const RegionInfo ni = decode_ticket(a, t, &next);
+                const int slot = (seq + 1) & 1;
+                const int4 *src = reinterpret_cast<const int4 *>(a.sims + ni.sim);
+                int4 *dst = reinterpret_cast<int4 *>(s_sd + slot);
+                if (lane < (int)(sizeof(SimDev) / 16)) dst[lane] = src[lane];
+                if (lane == 0) s_ri[slot] = ni;
+                __syncwarp();
+                const SimDev &nsd = s_sd[slot];
+                const TablesDev &T = s_tabs[nsd.tab_index];
+                f0 = pred_flag(a, nsd, T, ni, lane);
+                f1 = pred_flag(a, nsd, T, ni, lane + 32);
+                if (prefetch) prefetch_region_l2(nsd, T.type[ni.S], ni, lane);
+            }
+        }
+        if (!ready) {
+            const bool ok = (!f0 || ld_relaxed_gpu(f0) == epoch) && (!f1 || ld_relaxed_gpu(f1) == epoch);
+            ready = __all_sync(0xffffffffu, ok);
+            if (ready) {
+                fence_acq_rel_gpu();  // the predecessors' surfaces, read after the handoff below
+                __syncwarp();
+            } else if ((spin & 15u) == 15u) {
+                int stop = 0;
+                if (lane == 0) {
+                    if (ld_relaxed_gpu(&a.ctl->error) != 0) {
+                        stop = 1;
+                    } else if (globaltimer_ns() - t0 > limit) {
+                        atomicCAS(&a.ctl->error, 0, kDevTimeout);
+                        atomicExch(&a.ctl->error_info, (int)t);
+                        stop = 1;
+                    }
+                }
+                if (__shfl_sync(0xffffffffu, stop, 0)) {
+                    next = -2;
+                    ready = true;
+                }
+            }
+        }
+        int done = 0;
+        if (lane == 0) done = ld_acquire_cta_shared(s_done) == seq;
+        done = __shfl_sync(0xffffffffu, done, 0);
+        if (done && ready) {
+            if (lane == 0) {
+                s_slot[(seq + 1) & 1] = next;
+                st_release_cta_shared(s_handoff, seq + 1);
+            }
+            ++seq;
+            if (pending >= 0) report();
+            if (next < 0) break;
+            pending = next;
+            if (lane == 0) t = atomicAdd(&a.ctl->head, 1u);
+            t = __shfl_sync(0xffffffffu, t, 0);
+            staged = false;
+            t0 = globaltimer_ns();
+            t_progress = t0;
+            continue;
+        }
+        if (done && pending >= 0) {
+            report();
+            t_progress = globaltimer_ns();
+            continue;
+        }
+        // no handoff and no report for 4 wait limits: the worker is stuck;
+        // record it and stop (the worker's own bounded wait then ends it too)
+        int stuck = 0;
+        if (lane == 0 && (spin & 15u) == 15u && globaltimer_ns() - t_progress > 4 * limit) {
+            atomicCAS(&a.ctl->error, 0, kDevTimeout);
+            stuck = 1;
+        }
+        if (__shfl_sync(0xffffffffu, stuck, 0)) break;
+        // Waiting on the flags backs off: the polls share the SM's issue slots and L2
+        // with the working groups (32^3, base 4, 64 steps: 745 us at 32 ns, 671 at
+        // 300, 684 at 600; 48^3, base 8: 585, 536, 541).  Waiting on the worker polls
+        // shared memory.
+        if (!ready) __nanosleep(300);
+    }
+}
+
 // One instantiation per worker count NW, with the region base BB fixed at
 // compile time (16: index arithmetic in shifts, stencil offsets as immediates;
 // measured 1.5 % faster) or, for BB = 0, taken from the descriptor (bases 4
 // and 8, whose several CTAs per SM favour the smaller code: the fixed-base
 // build measured 1.4 % slower there).  A launch holds simulations of one base.
+// A CTA hosts `groups` regions at a time, each a group of a manager warp and NW
+// workers with its own buffers and named barrier, which share the tables and
+// import lists (base 8: 10.8 KB beside 25.3 KB a region, so eight regions fit
+// an SM where six CTAs did).  Bound by the latency of a level (import wait,
+// barrier, index, update, export: 0.8 us at base 16) times the levels a phase
+// chain holds, not by a pipe: 256^3, base 8, 8 steps 3.18 ms with six CTAs and
+// the ready queue, 3.04 ms with eight regions and tickets; 32^3, 64 steps 618 and
+// 434 us; 192^3, base 16, 64 steps 6.35 and 6.16 ms; 64^3 540 and 456 us.
 template <int NW, int BB>
-__global__ void __launch_bounds__(NW + 32, region_min_blocks(NW)) region_kernel(RegionArgs a, int max_P_launch)
+__global__ void __launch_bounds__(region_max_threads(NW), 1) region_kernel(RegionArgs a, int max_P_launch)
 {
     const int max_P = BB ? BB + 2 : max_P_launch;
     extern __shared__ __align__(16) unsigned char smem_raw[];
-    __shared__ int s_slot[2], s_handoff, s_done;
-    __shared__ SimDev s_sd[2];      // descriptor of the region handed over in each slot
-    __shared__ RegionInfo s_ri[2];  // and the region, decoded
-    __shared__ float2 *s_mb[64];  // consumer code (type | offset bits << 3) -> mailbox base
-    const int tid = threadIdx.x;
+    // Static, apart from the buffers, so that no store to a buffer can alias it.
+    // One region per CTA: a variable each at a constant address (as members of
+    // one struct they are 2.5 % slower at base 16); several: one struct each
+    // (an array of each member is 11 % slower at base 8, a base register more
+    // per array).
+    constexpr int G = region_max_groups(NW);
+    constexpr bool one = G == 1;
+    __shared__ GroupShared g_shared[G];
+    __shared__ int x_slot[2], x_handoff, x_done, x_abort;
+    __shared__ SimDev x_sd[2];
+    __shared__ RegionInfo x_ri[2];
+    __shared__ float2 *x_mb[64];
+    const int group = one ? 0 : threadIdx.x / (NW + 32), tid = threadIdx.x - group * (NW + 32);
+    const int kWorkerBarrier = 1 + group;
     const int P3 = max_P * max_P * max_P, B3 = (max_P - 2) * (max_P - 2) * (max_P - 2);
-    float2 *phi_buf0 = reinterpret_cast<float2 *>(smem_raw);
+    // one region: its buffers at constant offsets, then the tables; several: the tables first
+    const int groups = one ? 1 : blockDim.x / (NW + 32);
+    TablesDev *s_tabs = reinterpret_cast<TablesDev *>(smem_raw + (one ? region_group_bytes(max_P - 2) : 0));
+    unsigned char *const mine =
+        smem_raw + (one ? 0 : (size_t)a.n_tabs * sizeof(TablesDev) + (size_t)group * region_group_bytes(max_P - 2));
+    float2 *phi_buf0 = reinterpret_cast<float2 *>(mine);
     float2 *phi_buf1 = phi_buf0 + P3;
     float4 *pc_s = reinterpret_cast<float4 *>(phi_buf1 + P3);
-    TablesDev *s_tabs = reinterpret_cast<TablesDev *>(pc_s + B3);
-    LevelCoef *s_coef = reinterpret_cast<LevelCoef *>(s_tabs + a.n_tabs);
-
-    {  // the launch's tables and simulation descriptors, once
+    LevelCoef *s_coef = reinterpret_cast<LevelCoef *>(pc_s + B3);
+    {  // the launch's tables, once
         const int4 *src = reinterpret_cast<const int4 *>(a.tabs);
         int4 *dst = reinterpret_cast<int4 *>(s_tabs);
         const int nt = a.n_tabs * (int)(sizeof(TablesDev) / 16);
-        for (int i = tid; i < nt; i += NW + 32) dst[i] = src[i];
-        if (tid == 0) {
-            s_handoff = 0;
-            s_done = 0;
-        }
+        for (int i = threadIdx.x; i < nt; i += blockDim.x) dst[i] = src[i];
     }
     __syncthreads();
-    unsigned short *s_imp = reinterpret_cast<unsigned short *>(s_coef + kMaxHDev);
+    unsigned short *s_imp = reinterpret_cast<unsigned short *>(smem_raw + (size_t)a.n_tabs * sizeof(TablesDev) +
+                                                               (size_t)groups * region_group_bytes(max_P - 2));
     for (int t = 0; t < a.n_tabs; ++t) {  // every import list of the launch, once
         const int4 *src = reinterpret_cast<const int4 *>(s_tabs[t].imp);
         int4 *dst = reinterpret_cast<int4 *>(s_imp + s_tabs[t].imp_smem);
-        for (int i = tid; i < s_tabs[t].imp_n / 8; i += NW + 32) dst[i] = src[i];
+        for (int i = threadIdx.x; i < s_tabs[t].imp_n / 8; i += blockDim.x) dst[i] = src[i];
+    }
+    GroupShared &gs = g_shared[group];
+    int *const s_slot = one ? x_slot : gs.slot;
+    int &s_handoff = one ? x_handoff : gs.handoff, &s_done = one ? x_done : gs.done, &s_abort = one ? x_abort : gs.abort;
+    SimDev *const s_sd = one ? x_sd : gs.sd;
+    RegionInfo *const s_ri = one ? x_ri : gs.ri;
+    float2 **const s_mb = one ? x_mb : gs.mb;
+    if (tid == 0) {
+        s_handoff = 0;
+        s_done = 0;
     }
     __syncthreads();
     if (tid < 32) {
-        manager_loop(a, s_tabs, s_slot, s_sd, s_ri, &s_handoff, &s_done, BB == 16);
+        if (a.flags)
+            manager_tickets(a, s_tabs, s_slot, s_sd, s_ri, &s_handoff, &s_done, BB == 16);
+        else
+            manager_loop(a, s_tabs, s_slot, s_sd, s_ri, &s_handoff, &s_done, BB == 16);
         return;
     }
     const int wt = tid - 32;  // worker thread index
-    __shared__ int s_abort;
     for (int seq = 1;; ++seq) {
         if (wt == 0) {
             // bounded wait for the manager's handoff (a shared-memory poll: the
@@ -570,20 +793,33 @@ __global__ void __launch_bounds__(NW + 32, region_min_blocks(NW)) region_kernel(
             const int ne = k >= 2 ? M.exp_n[k - 1] : 0;
             const int2 *el = T.exp + (k >= 2 ? M.exp_off[k - 1] : 0);
             prefetch_entries<NW>(el, ne, pre, wt);
+            constexpr int U = region_cells_per_step(NW);
+            // bases 4 and 8: the level's box and the thread's next cells ahead of the
+            // barrier and of the updates (128^3, base 8: 5.79 ms, 6.03 without); at
+            // base 16 the registers they hold cost more than they hide (3.78, 3.72)
+            constexpr bool ahead = BB == 0;
+            int pidx[U], cidx[U];
+            LevelBox L;
+            if (ahead) {
+                L.load(M, k);
+                cell_indices<U>(wt, NW, L, P, B, pidx, cidx);
+            }
             cp_async_wait_pending(2);  // groups 0..k-1 (base, coefficients, levels < k) have landed
             named_barrier(kWorkerBarrier, NW);
             // ---- evolve the cells of level k, several independent cells per step ----
             const LevelCoef co = s_coef[k - 1];
-            const Box3 A = M.active[k];
-            const float rc = M.rcp_active[k][0], ra = M.rcp_active[k][1];
-            const int w0 = A.hi[0] - A.lo[0], w2 = A.hi[2] - A.lo[2];
-            const int cnt = w0 * (A.hi[1] - A.lo[1]) * w2;
-            const int a = w0 >> 1, cz = w2 >> 1;  // 2x2x2 blocks along x and z
+            if (!ahead) L.load(M, k);
             int i = wt;
-            constexpr int U = region_cells_per_step(NW);
-            for (; i + (U - 1) * NW < cnt; i += U * NW)
-                evolve_cells<U>(i, NW, A, a, cz, rc, ra, P, PP, B, prev_buf, cur, pc_s, co, q);
-            for (; i < cnt; i += NW) evolve_cell(i, A, a, cz, rc, ra, P, PP, B, prev_buf, cur, pc_s, co, q);
+            for (; i + (U - 1) * NW < L.cnt; i += U * NW) {
+                if (!ahead) cell_indices<U>(i, NW, L, P, B, pidx, cidx);
+                evolve_cells<U>(pidx, cidx, P, PP, prev_buf, cur, pc_s, co, q);
+                if (ahead) cell_indices<U>(i + U * NW, NW, L, P, B, pidx, cidx);
+            }
+            for (; U > 1 && i < L.cnt; i += NW) {  // fewer than U left
+                int p1[1], c1[1];
+                cell_indices<1>(i, NW, L, P, B, p1, c1);
+                evolve_cells<1>(p1, c1, P, PP, prev_buf, cur, pc_s, co, q);
+            }
             // ---- final surface of level k-1 (read-only data of level k-1) ----
             if (ne > 0) export_entries<NW>(el, ne, pre, s_mb, prev_buf, pc_s, wt);
         }
@@ -741,6 +977,10 @@ cudaError_t launch_features(const RegionArgs &a, const float4 *simf, const unsig
 
 cudaError_t launch_reset(const RegionArgs &a, cudaStream_t st)
 {
+    if (a.flags) {
+        ticket_reset_kernel<<<1, 1, 0, st>>>(a.ctl, a.epoch);
+        return cudaGetLastError();
+    }
     const unsigned blocks = (a.total + 255) / 256;
     reset_kernel<<<blocks ? blocks : 1, 256, 0, st>>>(a);
     if (a.prio && a.n_seed > 0) {
@@ -750,104 +990,64 @@ cudaError_t launch_reset(const RegionArgs &a, cudaStream_t st)
     return cudaGetLastError();
 }
 
-template <int NW, int BB>
-static cudaError_t region_launch_t(const RegionArgs &a, int B, size_t smem, int grid, cudaStream_t st)
+static const void *region_fn(int threads, int B)
 {
-    cudaError_t e =
-        cudaFuncSetAttribute(region_kernel<NW, BB>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e != cudaSuccess) return e;
-    region_kernel<NW, BB><<<grid, NW + 32, smem, st>>>(a, B + 2);
-    return cudaGetLastError();
-}
-
-template <int NW>
-static cudaError_t region_launch_nw(const RegionArgs &a, int B, size_t smem, int grid, cudaStream_t st)
-{
-    switch (B) {
-    case 4:
-    case 8:
-        return region_launch_t<NW, 0>(a, B, smem, grid, st);
-    case 16:
-        return region_launch_t<NW, 16>(a, B, smem, grid, st);
-    default:
-        return cudaErrorInvalidValue;
-    }
-}
-
-template <int NW, int BB>
-static cudaError_t region_occupancy_t(size_t smem, int *blocks_per_sm)
-{
-    cudaError_t e = cudaFuncSetAttribute(region_kernel<NW, BB>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e != cudaSuccess) return e;
-    return cudaOccupancyMaxActiveBlocksPerMultiprocessor(blocks_per_sm, region_kernel<NW, BB>, NW + 32, smem);
-}
-
-template <int NW>
-static cudaError_t region_occupancy_nw(int B, size_t smem, int *blocks_per_sm)
-{
-    switch (B) {
-    case 4:
-    case 8:
-        return region_occupancy_t<NW, 0>(smem, blocks_per_sm);
-    case 16:
-        return region_occupancy_t<NW, 16>(smem, blocks_per_sm);
-    default:
-        return cudaErrorInvalidValue;
-    }
-}
-
-size_t region_smem_bytes(int max_B, int n_tabs, int n_sims, int imp_units)
-{
-    (void)n_sims;  // descriptors travel with the handoff (static shared memory)
-    const int P = max_B + 2;
-    return (size_t)2 * P * P * P * sizeof(float2) + (size_t)max_B * max_B * max_B * sizeof(float4) +
-           (size_t)n_tabs * sizeof(TablesDev) + kMaxHDev * sizeof(LevelCoef) +
-           (size_t)imp_units * sizeof(unsigned short);
-}
-
-// threads = worker threads per CTA (the manager warp comes on top)
-cudaError_t region_occupancy(int threads, int B, size_t smem, int *blocks_per_sm)
-{
-#define SP_OCC(NW)                                                                                               \
-    case NW:                                                                                                     \
-        return region_occupancy_nw<NW>(B, smem, blocks_per_sm);
+    const bool b16 = B == 16;
+    if (B != 4 && B != 8 && B != 16) return nullptr;
     switch (threads) {
-        SP_OCC(64)
-        SP_OCC(128)
-        SP_OCC(256)
-        SP_OCC(320)
-        SP_OCC(384)
-        SP_OCC(480)
-        SP_OCC(512)
-        SP_OCC(768)
+#define SP_REGION(NW) \
+    case NW:          \
+        return b16 ? (const void *)region_kernel<NW, 16> : (const void *)region_kernel<NW, 0>;
+        SP_REGION(64)
+        SP_REGION(128)
+        SP_REGION(256)
+        SP_REGION(320)
+        SP_REGION(384)
+        SP_REGION(480)
+        SP_REGION(512)
+        SP_REGION(768)
+#undef SP_REGION
     default:
-        return cudaErrorInvalidValue;
+        return nullptr;
     }
-#undef SP_OCC
 }
 
-cudaError_t launch_region(const RegionArgs &a, int threads, int max_B, size_t smem, int grid, cudaStream_t st)
+// threads = worker threads per region (its manager warp comes on top)
+cudaError_t region_config(int threads, int B, int imp_units, RegionConfig *c)
 {
-    switch (threads) {
-    case 64:
-        return region_launch_nw<64>(a, max_B, smem, grid, st);
-    case 128:
-        return region_launch_nw<128>(a, max_B, smem, grid, st);
-    case 256:
-        return region_launch_nw<256>(a, max_B, smem, grid, st);
-    case 320:
-        return region_launch_nw<320>(a, max_B, smem, grid, st);
-    case 384:
-        return region_launch_nw<384>(a, max_B, smem, grid, st);
-    case 480:
-        return region_launch_nw<480>(a, max_B, smem, grid, st);
-    case 512:
-        return region_launch_nw<512>(a, max_B, smem, grid, st);
-    case 768:
-        return region_launch_nw<768>(a, max_B, smem, grid, st);
-    default:
-        return cudaErrorInvalidValue;
+    *c = RegionConfig();
+    const void *f = region_fn(threads, B);
+    if (!f) return cudaErrorInvalidValue;
+    cudaFuncAttributes fa;
+    cudaError_t e = cudaFuncGetAttributes(&fa, f);
+    if (e != cudaSuccess) return e;
+    // the number of regions per CTA that leaves the most of them on an SM
+    for (int g = 1; g <= region_max_groups(threads); ++g) {
+        const size_t smem = sizeof(TablesDev) + (size_t)imp_units * sizeof(unsigned short) + g * region_group_bytes(B);
+        if (smem + fa.sharedSizeBytes > 227 * 1024) break;
+        int ctas = 0;
+        e = cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&ctas, f, g * (threads + 32), smem);
+        if (e != cudaSuccess) return e;
+        if (ctas * g >= c->ctas_per_sm * c->groups) {
+            c->groups = g;
+            c->ctas_per_sm = ctas;
+            c->smem = smem;
+        }
     }
+    return cudaSuccess;
+}
+
+cudaError_t launch_region(const RegionArgs &a, int threads, int B, int groups, size_t smem, int grid, cudaStream_t st)
+{
+    const void *f = region_fn(threads, B);
+    if (!f) return cudaErrorInvalidValue;
+    cudaError_t e = cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    if (e != cudaSuccess) return e;
+    int P = B + 2;
+    void *args[2] = {const_cast<RegionArgs *>(&a), &P};
+    e = cudaLaunchKernel(f, dim3((unsigned)grid), dim3((unsigned)(groups * (threads + 32))), args, smem, st);
+    return e != cudaSuccess ? e : cudaGetLastError();
 }
 
 cudaError_t launch_sweep(const float2 *phi_in, float2 *phi_out, float4 *pc, const int n[3],
