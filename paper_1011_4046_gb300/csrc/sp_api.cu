@@ -570,9 +570,8 @@ int build_device_tables(sp_grid *g, int B)
         {
             const sp::Box3 &bp = t.base_phi[S];
             m.base_cols = (bp.hi[0] - bp.lo[0]) * (bp.hi[1] - bp.lo[1]);
-            m.base_runs = (bp.hi[2] - bp.lo[2] + 3) / 4;
             m.rcp_cols = 1.0f / (float)m.base_cols;
-            for (int u = 0; u < m.base_cols * m.base_runs; ++u)  // the kernel's (run, column) split
+            for (int u = 0; u < m.base_cols * (bp.hi[2] - bp.lo[2]); ++u)  // the kernel's (run, column) split
                 if (sp::fdiv(u, m.rcp_cols) != u / m.base_cols) return SP_EINVAL;
         }
         if (!block_decode_exact(m.active, t.H, m.rcp_active) || !decode_exact(&m.base_phi, 0, &m.rcp_base))

@@ -18,10 +18,12 @@ constexpr int kMaxHDev = 8;
 struct alignas(16) TypeMeta {
     int levels, mb_size, n_same_succ, same_preds;
     int prev_preds;
-    // band-base copy in units of (column, run of up to 4 cells along z):
-    // columns of the base box, runs per column, 1/columns in FP32
-    int base_cols, base_runs;
+    // band-base copy in units of (column, run of base_len cells along z):
+    // columns of the base box, 1/columns in FP32; the kernel chooses the run
+    // for its workers (base_len, and runs per column) in its own copy
+    int base_cols;
     float rcp_cols;
+    int base_len, base_runs;
     Box3 active[kMaxHDev + 1];
     Box3 base_phi, base_pc;
     // exact quotient decode (see fdiv below), reciprocals rounded to FP32:

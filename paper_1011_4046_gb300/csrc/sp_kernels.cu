@@ -145,6 +145,7 @@ static_assert(sizeof(SimDev) / 16 <= 32, "the manager warp copies a descriptor w
 // read in batches.  Three cover the average level of base 16 with 256
 // workers several times over; more cost registers and unrolled code for
 // entries that rarely exist.
+constexpr int kBaseRun = 4;  // most cells of a unit of the base copy
 constexpr int kExportPrefetch = 3;
 constexpr int kExportBatch = 4;
 // Per worker count: independent cell updates in flight per thread (measured:
@@ -157,7 +158,8 @@ __host__ __device__ constexpr int region_cells_per_step(int nw) { return nw <= 1
 // Most threads of a CTA (workers and manager warps of its groups), which set the
 // register budget: eight regions of 64 workers, four of 128, one of more.
 __host__ __device__ constexpr int region_max_groups(int nw) { return nw <= 64 ? 8 : nw <= 128 ? 4 : 1; }
-__host__ __device__ constexpr int region_max_threads(int nw) { return region_max_groups(nw) * (nw + 32); }
+__host__ __device__ constexpr int region_reporter(int nw) { return nw > 64 ? 32 : 0; }  // threads
+__host__ __device__ constexpr int region_max_threads(int nw) { return region_max_groups(nw) * (nw + 32) + region_reporter(nw); }
 
 // What one of several groups shares beside its buffers: descriptor and decoded
 // region of each handoff slot, mailbox base by consumer code (type | offset bits
@@ -166,7 +168,7 @@ struct alignas(16) GroupShared {
     SimDev sd[2];
     RegionInfo ri[2];
     float2 *mb[64];
-    int slot[2], handoff, done, abort;
+    int slot[4], handoff, done, reported, last, abort;
 };
 
 __host__ __device__ constexpr size_t region_group_bytes(int B)
@@ -413,7 +415,7 @@ __device__ void manager_loop(const RegionArgs &a, const TablesDev *s_tabs, int *
         done = __shfl_sync(0xffffffffu, done, 0);
         if (done && have) {
             if (lane == 0) {
-                s_slot[(seq + 1) & 1] = next;
+                s_slot[(seq + 1) & 3] = next;
                 st_release_cta_shared(s_handoff, seq + 1);
             }
             ++seq;
@@ -503,117 +505,159 @@ __device__ __forceinline__ const int *pred_flag(const RegionArgs &a, const SimDe
     return a.flags + (sd.tile_base + (unsigned)((band * 8 + (p.type_prev & 7)) * sd.Jtot + jc));
 }
 
+// What a group's manager, its worker and the reporter warp share: the regions
+// handed over (by count mod 4), finished and reported so far, and how many there
+// will be (-1: not known).
+struct GroupSync {
+    int *slot, *handoff, *done, *reported, *last;
+};
+
+// Sets the done flag of the group's next finished region, if there is one past
+// the first seq: the release orders the worker's surfaces (its done count is
+// acquired) before the flag.
+__device__ __forceinline__ bool report_next(const RegionArgs &a, int epoch, const GroupSync &y, int seq)
+{
+    if (ld_acquire_cta_shared(y.done) <= seq) return false;
+    const int g = y.slot[(seq + 1) & 3];
+    if (g != a.fault_drop) st_release_gpu(a.flags + g, epoch);
+    return true;
+}
+
 // Manager warp in ticket order: takes the next ticket, stages its region while
 // the worker evolves the current one, polls the done flags of the region's
-// predecessors (two per lane), hands it over, and reports the finished region
-// by its own flag.  No queue and no counters: a release is one fence and one
-// store where decrementing every successor and pushing the ready ones took
-// about 3 us, as long as a base-8 region, and all managers shared the queue's
-// head and tail.  Tickets are taken in a topological order and every ticket is
-// held by a resident manager whose worker has only smaller ones before it,
-// so the waits end; each is bounded anyway.
-__device__ void manager_tickets(const RegionArgs &a, const TablesDev *s_tabs, int *s_slot, SimDev *s_sd, RegionInfo *s_ri,
-                                int *s_handoff, int *s_done, bool prefetch)
+// predecessors (two per lane) and hands it over, before the worker has finished
+// if it can, so that the worker goes from one region to the next by itself.  No
+// queue and no counters: a release is one store where decrementing every
+// successor and pushing the ready ones took about 3 us, as long as a base-8
+// region, and all managers shared the queue's head and tail.  Tickets are taken
+// in a topological order and every ticket is held by a resident manager whose
+// worker has only smaller ones before it, so the waits end; each is bounded
+// anyway.  Polls that acquire and stores that release, not relaxed ones with
+// fences: a fence waits about a microsecond in either place (32^3, base 8, 64
+// steps: 401 us with a fence at both ends, 380 without).
+// OWN: the manager also reports (64 workers, where a CTA has no room for
+// the reporter warp).
+template <bool OWN>
+__device__ void manager_tickets(const RegionArgs &a, const TablesDev *s_tabs, SimDev *s_sd, RegionInfo *s_ri,
+                                const GroupSync &y, bool prefetch)
 {
     const int lane = threadIdx.x & 31;
     const unsigned long long limit = a.ctl->wait_limit_ns;
     const int epoch = *(volatile int *)a.epoch;
-    int seq = 0;       // handoffs made
-    int pending = -1;  // region handed at seq, not yet reported
-    unsigned t = 0;
-    if (lane == 0) t = atomicAdd(&a.ctl->head, 1u);
-    t = __shfl_sync(0xffffffffu, t, 0);
-    int next = -1;     // region of ticket t, staged; -1: no more, -2: stop
-    bool staged = false, ready = false;
-    const int *f0 = nullptr, *f1 = nullptr;
-    unsigned long long t0 = globaltimer_ns(), t_progress = t0;
-    auto report = [&]() {
-        if (lane == 0 && pending != a.fault_drop) {
-            fence_acq_rel_gpu();  // the worker's surfaces (its done flag was acquired) before the region's flag
-            st_relaxed_gpu(a.flags + pending, epoch);
-        }
-        pending = -1;
-    };
-    for (unsigned spin = 0;; ++spin) {
-        if (!staged) {
-            staged = true;
-            ready = t >= a.total;
-            next = -1;
-            if (!ready) {
-                const RegionInfo ni = decode_ticket(a, t, &next);
-                const int slot = (seq + 1) & 1;
-                const int4 *src = reinterpret_cast<const int4 *>(a.sims + ni.sim);
-                int4 *dst = reinterpret_cast<int4 *>(s_sd + slot);
-                if (lane < (int)(sizeof(SimDev) / 16)) dst[lane] = src[lane];
-                if (lane == 0) s_ri[slot] = ni;
-                __syncwarp();
-                const SimDev &nsd = s_sd[slot];
-                const TablesDev &T = s_tabs[nsd.tab_index];
-                f0 = pred_flag(a, nsd, T, ni, lane);
-                f1 = pred_flag(a, nsd, T, ni, lane + 32);
-                if (prefetch) prefetch_region_l2(nsd, T.type[ni.S], ni, lane);
+    int seq = 0, reported = 0;  // handoffs made; OWN, lane 0: regions reported
+    // lane 0 waits for the worker to have finished n regions (and for the last but
+    // two of them to be reported: there are four id slots); false: it is stuck
+    auto finished = [&](int n) {
+        unsigned long long t0 = 0;
+        for (unsigned spin = 0;; ++spin) {
+            if (OWN)
+                reported += report_next(a, epoch, y, reported);
+            if (OWN ? reported >= n
+                    : ld_acquire_cta_shared(y.done) >= n && ld_acquire_cta_shared(y.reported) >= n - 2)
+                return true;
+            if ((spin & 63u) == 63u) {
+                if (t0 == 0) t0 = globaltimer_ns();
+                if (globaltimer_ns() - t0 > 4 * limit) {
+                    atomicCAS(&a.ctl->error, 0, kDevTimeout);
+                    return false;
+                }
             }
         }
-        if (!ready) {
-            const bool ok = (!f0 || ld_relaxed_gpu(f0) == epoch) && (!f1 || ld_relaxed_gpu(f1) == epoch);
-            ready = __all_sync(0xffffffffu, ok);
-            if (ready) {
-                fence_acq_rel_gpu();  // the predecessors' surfaces, read after the handoff below
-                __syncwarp();
-            } else if ((spin & 15u) == 15u) {
-                int stop = 0;
-                if (lane == 0) {
-                    if (ld_relaxed_gpu(&a.ctl->error) != 0) {
-                        stop = 1;
-                    } else if (globaltimer_ns() - t0 > limit) {
-                        atomicCAS(&a.ctl->error, 0, kDevTimeout);
-                        atomicExch(&a.ctl->error_info, (int)t);
-                        stop = 1;
+    };
+    for (;;) {
+        // the descriptor slot of the region before the current one
+        bool stop = false;
+        unsigned t = 0;
+        if (lane == 0) {
+            stop = !finished(seq - 1);
+            if (!stop) t = atomicAdd(&a.ctl->head, 1u);
+        }
+        stop = __shfl_sync(0xffffffffu, stop, 0);
+        t = __shfl_sync(0xffffffffu, t, 0);
+        int next = stop ? -2 : -1;  // region handed over; -1: no more, -2: stop
+        if (!stop && t < a.total) {
+            const RegionInfo ni = decode_ticket(a, t, &next);
+            const int slot = (seq + 1) & 1;
+            const int4 *src = reinterpret_cast<const int4 *>(a.sims + ni.sim);
+            int4 *dst = reinterpret_cast<int4 *>(s_sd + slot);
+            if (lane < (int)(sizeof(SimDev) / 16)) dst[lane] = src[lane];
+            if (lane == 0) s_ri[slot] = ni;
+            __syncwarp();
+            const SimDev &nsd = s_sd[slot];
+            const TablesDev &T = s_tabs[nsd.tab_index];
+            const int *f0 = pred_flag(a, nsd, T, ni, lane), *f1 = pred_flag(a, nsd, T, ni, lane + 32);
+            const unsigned long long t0 = globaltimer_ns();
+            for (unsigned spin = 0;; ++spin) {
+                if (f0 && ld_acquire_gpu(f0) == epoch) f0 = nullptr;
+                if (f1 && ld_acquire_gpu(f1) == epoch) f1 = nullptr;
+                const bool ok = !f0 && !f1;
+                if (__all_sync(0xffffffffu, ok)) break;
+                if (OWN && lane == 0) reported += report_next(a, epoch, y, reported);
+                if ((spin & 15u) == 15u) {
+                    if (lane == 0) {
+                        if (ld_relaxed_gpu(&a.ctl->error) != 0) {
+                            stop = true;
+                        } else if (globaltimer_ns() - t0 > limit) {
+                            atomicCAS(&a.ctl->error, 0, kDevTimeout);
+                            atomicExch(&a.ctl->error_info, (int)t);
+                            stop = true;
+                        }
+                    }
+                    stop = __shfl_sync(0xffffffffu, stop, 0);
+                    if (stop) {
+                        next = -2;
+                        break;
                     }
                 }
-                if (__shfl_sync(0xffffffffu, stop, 0)) {
-                    next = -2;
-                    ready = true;
-                }
+                // The polls share the SM's issue slots and L2 with the working groups, and
+                // an acquire empties L1 (32^3, base 4, 64 steps: 642 us at 100 ns, 562 at
+                // 300, 565 at 500; 48^3, base 8: 521, 456, 454; 545 and 444 at 300 since a
+                // lane leaves out what it has seen).
+                __nanosleep(300);
+            }
+            __syncwarp();  // every lane's acquire before lane 0's release below
+        }
+        if (lane == 0) {
+            y.slot[(seq + 1) & 3] = next;
+            if (next < 0) st_release_cta_shared(y.last, seq);
+            st_release_cta_shared(y.handoff, seq + 1);
+        }
+        if (next < 0) {
+            if (OWN && lane == 0) finished(seq);
+            break;
+        }
+        ++seq;
+        if (prefetch) {
+            const SimDev &nsd = s_sd[seq & 1];
+            prefetch_region_l2(nsd, s_tabs[nsd.tab_index].type[s_ri[seq & 1].S], s_ri[seq & 1], lane);
+        }
+    }
+}
+
+// Reporter warp of a CTA: lane g sets the done flag of each region that group g
+// has finished.  A warp of its own, so that a flag waits for no manager's staging
+// or poll (48^3, base 8, 64 steps: 488 us with reporting managers, 455).
+__device__ void report_regions(const RegionArgs &a, int groups, const GroupSync &y)
+{
+    const int lane = threadIdx.x & 31;
+    const int epoch = *(volatile int *)a.epoch;
+    const unsigned long long limit = 16 * a.ctl->wait_limit_ns;
+    unsigned long long t0 = globaltimer_ns();
+    int seq = 0;  // regions reported
+    bool live = lane < groups;
+    for (unsigned spin = 0; __any_sync(0xffffffffu, live); ++spin) {
+        if (live) {
+            const int last = ld_acquire_cta_shared(y.last);
+            if (report_next(a, epoch, y, seq)) {
+                st_release_cta_shared(y.reported, ++seq);
+                t0 = globaltimer_ns();
+            } else if (last >= 0 && seq >= last) {
+                live = false;
+            } else if ((spin & 255u) == 255u &&
+                       ((last >= 0 && ld_relaxed_gpu(&a.ctl->error) != 0) || globaltimer_ns() - t0 > limit)) {
+                live = false;  // the launch has failed
             }
         }
-        int done = 0;
-        if (lane == 0) done = ld_acquire_cta_shared(s_done) == seq;
-        done = __shfl_sync(0xffffffffu, done, 0);
-        if (done && ready) {
-            if (lane == 0) {
-                s_slot[(seq + 1) & 1] = next;
-                st_release_cta_shared(s_handoff, seq + 1);
-            }
-            ++seq;
-            if (pending >= 0) report();
-            if (next < 0) break;
-            pending = next;
-            if (lane == 0) t = atomicAdd(&a.ctl->head, 1u);
-            t = __shfl_sync(0xffffffffu, t, 0);
-            staged = false;
-            t0 = globaltimer_ns();
-            t_progress = t0;
-            continue;
-        }
-        if (done && pending >= 0) {
-            report();
-            t_progress = globaltimer_ns();
-            continue;
-        }
-        // no handoff and no report for 4 wait limits: the worker is stuck;
-        // record it and stop (the worker's own bounded wait then ends it too)
-        int stuck = 0;
-        if (lane == 0 && (spin & 15u) == 15u && globaltimer_ns() - t_progress > 4 * limit) {
-            atomicCAS(&a.ctl->error, 0, kDevTimeout);
-            stuck = 1;
-        }
-        if (__shfl_sync(0xffffffffu, stuck, 0)) break;
-        // Waiting on the flags backs off: the polls share the SM's issue slots and L2
-        // with the working groups (32^3, base 4, 64 steps: 745 us at 32 ns, 671 at
-        // 300, 684 at 600; 48^3, base 8: 585, 536, 541).  Waiting on the worker polls
-        // shared memory.
-        if (!ready) __nanosleep(300);
     }
 }
 
@@ -625,11 +669,14 @@ __device__ void manager_tickets(const RegionArgs &a, const TablesDev *s_tabs, in
 // A CTA hosts `groups` regions at a time, each a group of a manager warp and NW
 // workers with its own buffers and named barrier, which share the tables and
 // import lists (base 8: 10.8 KB beside 25.3 KB a region, so eight regions fit
-// an SM where six CTAs did).  Bound by the latency of a level (import wait,
-// barrier, index, update, export: 0.8 us at base 16) times the levels a phase
-// chain holds, not by a pipe: 256^3, base 8, 8 steps 3.18 ms with six CTAs and
-// the ready queue, 3.04 ms with eight regions and tickets; 32^3, 64 steps 618 and
-// 434 us; 192^3, base 16, 64 steps 6.35 and 6.16 ms; 64^3 540 and 456 us.
+// an SM where six CTAs did).  Bound by latency, not by a pipe: at base 16 a
+// region takes 6.7 to 11 us, 0.8 us to request its base, 0.4 to wait for it and
+// 0.6 a level (import wait, barrier, index, update, export; 0.2 of it the
+// updates); 40 % of the issue slots and 28 % of DRAM are used (base 8: 62 and
+// 34 %).  On a small grid the hop from a region to its successor adds 2 us.
+// With the ready queue, and six CTAs at base 8, against this: 256^3, base 8, 8
+// steps 3.18 and 3.04 ms; 32^3, 64 steps 618 and 334 us; 192^3, base 16, 64
+// steps 6.35 and 6.13 ms; 64^3 540 and 425 us.
 template <int NW, int BB>
 __global__ void __launch_bounds__(region_max_threads(NW), 1) region_kernel(RegionArgs a, int max_P_launch)
 {
@@ -643,15 +690,15 @@ __global__ void __launch_bounds__(region_max_threads(NW), 1) region_kernel(Regio
     constexpr int G = region_max_groups(NW);
     constexpr bool one = G == 1;
     __shared__ GroupShared g_shared[G];
-    __shared__ int x_slot[2], x_handoff, x_done, x_abort;
+    __shared__ int x_slot[4], x_handoff, x_done, x_reported, x_last, x_abort;
     __shared__ SimDev x_sd[2];
     __shared__ RegionInfo x_ri[2];
     __shared__ float2 *x_mb[64];
+    const int groups = one ? 1 : blockDim.x / (NW + 32);  // and the reporter warp
     const int group = one ? 0 : threadIdx.x / (NW + 32), tid = threadIdx.x - group * (NW + 32);
     const int kWorkerBarrier = 1 + group;
     const int P3 = max_P * max_P * max_P, B3 = (max_P - 2) * (max_P - 2) * (max_P - 2);
     // one region: its buffers at constant offsets, then the tables; several: the tables first
-    const int groups = one ? 1 : blockDim.x / (NW + 32);
     TablesDev *s_tabs = reinterpret_cast<TablesDev *>(smem_raw + (one ? region_group_bytes(max_P - 2) : 0));
     unsigned char *const mine =
         smem_raw + (one ? 0 : (size_t)a.n_tabs * sizeof(TablesDev) + (size_t)group * region_group_bytes(max_P - 2));
@@ -668,12 +715,21 @@ __global__ void __launch_bounds__(region_max_threads(NW), 1) region_kernel(Regio
     __syncthreads();
     unsigned short *s_imp = reinterpret_cast<unsigned short *>(smem_raw + (size_t)a.n_tabs * sizeof(TablesDev) +
                                                                (size_t)groups * region_group_bytes(max_P - 2));
+    for (int t = threadIdx.x; t < kTypes * a.n_tabs; t += blockDim.x) {  // the shortest runs that give each worker one
+        TypeMeta &m = s_tabs[t / kTypes].type[t % kTypes];
+        const int w2 = m.base_phi.hi[2] - m.base_phi.lo[2];
+        int len = 1;
+        while (len < kBaseRun && m.base_cols * ((w2 + len - 1) / len) > NW) ++len;
+        m.base_len = len;
+        m.base_runs = (w2 + len - 1) / len;
+    }
     for (int t = 0; t < a.n_tabs; ++t) {  // every import list of the launch, once
         const int4 *src = reinterpret_cast<const int4 *>(s_tabs[t].imp);
         int4 *dst = reinterpret_cast<int4 *>(s_imp + s_tabs[t].imp_smem);
         for (int i = threadIdx.x; i < s_tabs[t].imp_n / 8; i += blockDim.x) dst[i] = src[i];
     }
-    GroupShared &gs = g_shared[group];
+    const bool reporter = region_reporter(NW) && threadIdx.x >= groups * (NW + 32);
+    GroupShared &gs = g_shared[reporter ? min(threadIdx.x & 31, groups - 1) : group];  // the reporter's lanes: a group each
     int *const s_slot = one ? x_slot : gs.slot;
     int &s_handoff = one ? x_handoff : gs.handoff, &s_done = one ? x_done : gs.done, &s_abort = one ? x_abort : gs.abort;
     SimDev *const s_sd = one ? x_sd : gs.sd;
@@ -682,11 +738,18 @@ __global__ void __launch_bounds__(region_max_threads(NW), 1) region_kernel(Regio
     if (tid == 0) {
         s_handoff = 0;
         s_done = 0;
+        (one ? x_reported : gs.reported) = 0;
+        (one ? x_last : gs.last) = -1;
     }
     __syncthreads();
+    const GroupSync sync = {s_slot, &s_handoff, &s_done, one ? &x_reported : &gs.reported, one ? &x_last : &gs.last};
+    if (reporter) {
+        if (a.flags) report_regions(a, groups, sync);
+        return;
+    }
     if (tid < 32) {
         if (a.flags)
-            manager_tickets(a, s_tabs, s_slot, s_sd, s_ri, &s_handoff, &s_done, BB == 16);
+            manager_tickets<region_reporter(NW) == 0>(a, s_tabs, s_sd, s_ri, sync, BB == 16);
         else
             manager_loop(a, s_tabs, s_slot, s_sd, s_ri, &s_handoff, &s_done, BB == 16);
         return;
@@ -697,18 +760,21 @@ __global__ void __launch_bounds__(region_max_threads(NW), 1) region_kernel(Regio
             // bounded wait for the manager's handoff (a shared-memory poll: the
             // handoff normally follows within a microsecond)
             s_abort = 0;
-            const unsigned long long t0 = globaltimer_ns(), limit = 8 * a.ctl->wait_limit_ns;
+            unsigned long long t0 = 0;
             for (unsigned spin = 0; ld_acquire_cta_shared(&s_handoff) < seq; ++spin) {
-                if ((spin & 15u) == 15u && globaltimer_ns() - t0 > limit) {
-                    atomicCAS(&a.ctl->error, 0, kDevTimeout);
-                    s_abort = 1;
-                    break;
+                if ((spin & 63u) == 63u) {
+                    if (t0 == 0) t0 = globaltimer_ns();
+                    if (globaltimer_ns() - t0 > 8 * a.ctl->wait_limit_ns) {
+                        atomicCAS(&a.ctl->error, 0, kDevTimeout);
+                        s_abort = 1;
+                        break;
+                    }
                 }
             }
         }
         named_barrier(kWorkerBarrier, NW);
         if (s_abort) break;
-        const int g = s_slot[seq & 1];
+        const int g = s_slot[seq & 3];
         if (g < 0) break;
         if (a.trace && wt == 0) a.trace[2 * (size_t)g] = globaltimer_ns();
 
@@ -737,15 +803,18 @@ __global__ void __launch_bounds__(region_max_threads(NW), 1) region_kernel(Regio
         }
 
         // ---- group 0: the band base (tops of the previous band) + coefficients ----
-        // Work units are (run of up to 4 cells along z, column), columns fastest:
+        // Work units are (run of base_len cells along z, column), columns fastest:
         // every worker gets a similar share whatever the box's shape, and
-        // consecutive threads read consecutive cells along x.
+        // consecutive threads read consecutive cells along x.  A run's cells are
+        // independent straight-line code: of the first microsecond of a region
+        // most was one warp's chain through runs of four while others had none
+        // (base 16, types 3 5 6 7: 0.68 us to the last request).
         {
             if (wt < H) cp_async16(s_coef + wt, sd.coef + band * H + wt);
             const Box3 bp = M.base_phi;
             const Box3 bc = M.base_pc;
             const int w0 = bp.hi[0] - bp.lo[0];
-            const int ncol = M.base_cols, units = ncol * M.base_runs;
+            const int ncol = M.base_cols, len = M.base_len, units = ncol * M.base_runs;
             for (int u = wt; u < units; u += NW) {
                 const int run = fdiv(u, M.rcp_cols);
                 const int i = u - run * ncol;
@@ -753,16 +822,19 @@ __global__ void __launch_bounds__(region_max_threads(NW), 1) region_kernel(Regio
                 const int ux = bp.lo[0] + i - t1 * w0;
                 const int uy = bp.lo[1] + t1;
                 const int oxy = (ux < bc.lo[0] || ux >= bc.hi[0]) + (uy < bc.lo[1] || uy >= bc.hi[1]);
-                if (oxy > 1) continue;  // not a 7-point neighbour of A(1)
                 const long long gxy =
                     (long long)wrap_axis(gbase[0] + ux, nx) + (long long)nx * wrap_axis(gbase[1] + uy, ny);
-                const int z0 = bp.lo[2] + 4 * run, z1 = min(z0 + 4, bp.hi[2]);
-                for (int uz = z0; uz < z1; ++uz) {
+                const int z0 = bp.lo[2] + len * run;
+#pragma unroll
+                for (int e = 0; e < kBaseRun; ++e) {
+                    const int uz = z0 + e;
+                    // out > 1: not a 7-point neighbour of A(1)
                     const int out = oxy + (uz < bc.lo[2] || uz >= bc.hi[2]);
-                    if (out > 1) continue;
                     const long long gi = gxy + nxy * wrap_axis(gbase[2] + uz, nz);
-                    cp_async8(phi_buf0 + (uz * P + uy) * P + ux, sd.phi + gi);
-                    if (out == 0) cp_async16(pc_s + pc_slot_of(ux, uy, uz, B), sd.pc + gi);
+                    if (e < len && uz < bp.hi[2] && out <= 1) {
+                        cp_async8(phi_buf0 + (uz * P + uy) * P + ux, sd.phi + gi);
+                        if (out == 0) cp_async16(pc_s + pc_slot_of(ux, uy, uz, B), sd.pc + gi);
+                    }
                 }
             }
             cp_async_commit();
@@ -834,17 +906,22 @@ __global__ void __launch_bounds__(region_max_threads(NW), 1) region_kernel(Regio
         } else {
             named_barrier(kWorkerBarrier, NW);
             // ---- tops of the inverted pyramid: the next band's base ----
-            const float rB = T.type[0].rcp_base[0];  // the pyramid's base box is B wide: 1/B
-            for (int i = wt; i < B * B; i += NW) {
-                const int t1 = fdiv(i, rB);
-                const int ux = 1 + i - t1 * B;
-                const int uy = 1 + t1;
+            const int lgB = 31 - __clz(B), share = B * B * B / NW;
+            const int len = share >= 4 ? 4 : share >= 2 ? 2 : 1;  // cells of a unit along z
+            for (int u = wt; u < B * B * B / len; u += NW) {
+                const int ux = 1 + (u & (B - 1));
+                const int uy = 1 + ((u >> lgB) & (B - 1));
+                const int z0 = 1 + len * (u >> (2 * lgB));
                 const long long gxy =
                     (long long)wrap_axis(gbase[0] + ux, nx) + (long long)nx * wrap_axis(gbase[1] + uy, ny);
-                for (int uz = 1; uz <= B; ++uz) {
+#pragma unroll
+                for (int e = 0; e < 4; ++e) {
+                    const int uz = z0 + e;
                     const long long gi = gxy + nxy * wrap_axis(gbase[2] + uz, nz);
-                    __stcg(sd.phi + gi, last[(uz * P + uy) * P + ux]);
-                    __stcg(sd.pc + gi, pc_s[pc_slot_of(ux, uy, uz, B)]);
+                    if (e < len) {
+                        __stcg(sd.phi + gi, last[(uz * P + uy) * P + ux]);
+                        __stcg(sd.pc + gi, pc_s[pc_slot_of(ux, uy, uz, B)]);
+                    }
                 }
             }
         }
@@ -1027,7 +1104,7 @@ cudaError_t region_config(int threads, int B, int imp_units, RegionConfig *c)
         if (smem + fa.sharedSizeBytes > 227 * 1024) break;
         int ctas = 0;
         e = cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-        if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&ctas, f, g * (threads + 32), smem);
+        if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&ctas, f, g * (threads + 32) + region_reporter(threads), smem);
         if (e != cudaSuccess) return e;
         if (ctas * g >= c->ctas_per_sm * c->groups) {
             c->groups = g;
@@ -1046,7 +1123,7 @@ cudaError_t launch_region(const RegionArgs &a, int threads, int B, int groups, s
     if (e != cudaSuccess) return e;
     int P = B + 2;
     void *args[2] = {const_cast<RegionArgs *>(&a), &P};
-    e = cudaLaunchKernel(f, dim3((unsigned)grid), dim3((unsigned)(groups * (threads + 32))), args, smem, st);
+    e = cudaLaunchKernel(f, dim3((unsigned)grid), dim3((unsigned)(groups * (threads + 32) + region_reporter(threads))), args, smem, st);
     return e != cudaSuccess ? e : cudaGetLastError();
 }
 
