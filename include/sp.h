@@ -213,7 +213,7 @@ int sp_grid_create(const sp_params *p, int32_t n_sims, void *const *state_dev, v
  *                s = 5, 512 at s = 6);
  *                every worker taking every step of a region); one manager
  *                warp is added.  0 for the default of each base (64 for
- *                base 4; 384 for 16; for 8, by the regions of a type on an SM,
+ *                base 4; 480 for 16; for 8, by the regions of a type on an SM,
  *                64; 128 up to five, 256 up to a half); SP_AUTOTUNE to time the
  *                candidates for the largest base (64, 128, 256 for base 8; 320,
  *                384, 480 for base 16), smaller bases keeping their default.

@@ -275,40 +275,6 @@ int check_params(const sp_params &p)
     return SP_OK;
 }
 
-// The kernel splits a linear index i < w0 w1 w2 into (x, y, z) with
-// sp::fdiv and FP32 reciprocals; check every quotient it will form.
-bool decode_exact(const sp::Box3 *boxes, int last, const float (*rcp)[2])
-{
-    for (int k = 0; k <= last; ++k) {
-        const sp::Box3 &b = boxes[k];
-        const int w0 = b.hi[0] - b.lo[0], w1 = b.hi[1] - b.lo[1], w2 = b.hi[2] - b.lo[2];
-        if (w0 <= 0 || w1 <= 0 || w2 <= 0) continue;
-        for (int i = 0; i < w0 * w1 * w2; ++i) {
-            const int t1 = sp::fdiv(i, rcp[k][0]);
-            if (t1 != i / w0 || sp::fdiv(t1, rcp[k][1]) != t1 / w1) return false;
-        }
-    }
-    return true;
-}
-
-// The same for the 2x2x2-block decode of the active boxes: block index
-// m < (w0/2)(w1/2)(w2/2) -> (m / (w2/2)) / (w0/2); every extent must be even.
-bool block_decode_exact(const sp::Box3 *boxes, int last, const float (*rcp)[2])
-{
-    for (int k = 0; k <= last; ++k) {
-        const sp::Box3 &b = boxes[k];
-        const int w0 = b.hi[0] - b.lo[0], w1 = b.hi[1] - b.lo[1], w2 = b.hi[2] - b.lo[2];
-        if (w0 <= 0 || w1 <= 0 || w2 <= 0) continue;
-        if ((w0 | w1 | w2) & 1) return false;
-        const int a = w0 / 2, c = w2 / 2;
-        for (int m = 0; m < a * (w1 / 2) * c; ++m) {
-            const int r = sp::fdiv(m, rcp[k][0]);
-            if (r != m / c || sp::fdiv(r, rcp[k][1]) != r / a) return false;
-        }
-    }
-    return true;
-}
-
 // The dependency pattern of a base (same-band, next-band and mailbox-reuse
 // successors, predecessor counts) into the device descriptor; geometry
 // fields are left to the caller.
@@ -557,32 +523,41 @@ int build_device_tables(sp_grid *g, int B)
         m.prev_preds = t.prev_preds[S];
         m.n_reuse = (int)t.reuse_succ[S].size();
         m.reuse_preds = t.reuse_preds[S];
-        for (int k = 0; k <= sp::kMaxHDev; ++k) m.active[k] = t.active[S][k];
         m.base_phi = t.base_phi[S];
         m.base_pc = t.base_pc[S];
-        for (int k = 0; k <= sp::kMaxHDev; ++k)
-            for (int q = 0; q < 2; ++q) {
-                const int d = q == 0 ? 2 : 0;  // blocks along z, then along x
-                const int w = (t.active[S][k].hi[d] - t.active[S][k].lo[d]) / 2;
-                m.rcp_active[k][q] = w > 0 ? 1.0f / (float)w : 0.0f;
+        for (int k = 0; k <= sp::kMaxHDev; ++k) {
+            const sp::Box3 &A = t.active[S][k];
+            const int w0 = A.hi[0] - A.lo[0], w1 = A.hi[1] - A.lo[1], w2 = A.hi[2] - A.lo[2];
+            if (w0 <= 0 || w1 <= 0 || w2 <= 0) continue;
+            sp::LevelBox &l = m.box[k];
+            for (int d = 0; d < 3; ++d) l.lo[d] = A.lo[d];
+            l.cnt = w0 * w1 * w2;
+            l.a = w0 / 2;
+            l.c = w2 / 2;
+            l.rc = sp::mdiv_mul(l.c);
+            l.ra = sp::mdiv_mul(l.a);
+            if ((w0 | w1 | w2) & 1) return SP_EINVAL;
+            for (int i = 0; i < l.a * (w1 / 2) * l.c; ++i) {  // the kernel's block decode
+                const int r = sp::mdiv(i, l.rc);
+                if (r != i / l.c || sp::mdiv(r, l.ra) != r / l.a) return SP_EINVAL;
             }
-        for (int d = 0; d < 2; ++d) m.rcp_base[d] = 1.0f / (float)(t.base_phi[S].hi[d] - t.base_phi[S].lo[d]);
+        }
         {
             const sp::Box3 &bp = t.base_phi[S];
             m.base_cols = (bp.hi[0] - bp.lo[0]) * (bp.hi[1] - bp.lo[1]);
-            m.rcp_cols = 1.0f / (float)m.base_cols;
-            for (int u = 0; u < m.base_cols * (bp.hi[2] - bp.lo[2]); ++u)  // the kernel's (run, column) split
-                if (sp::fdiv(u, m.rcp_cols) != u / m.base_cols) return SP_EINVAL;
+            const int w0 = bp.hi[0] - bp.lo[0];
+            m.mul_cols = sp::mdiv_mul(m.base_cols);
+            m.mul_w0 = sp::mdiv_mul(w0);
+            for (int u = 0; u < m.base_cols * (bp.hi[2] - bp.lo[2]); ++u) {  // the kernel's (run, column, row) split
+                const int i = u % m.base_cols;
+                if (sp::mdiv(u, m.mul_cols) != u / m.base_cols || sp::mdiv(i, m.mul_w0) != i / w0) return SP_EINVAL;
+            }
         }
-        if (!block_decode_exact(m.active, t.H, m.rcp_active) || !decode_exact(&m.base_phi, 0, &m.rcp_base))
-            return SP_EINVAL;
         for (int L = 0; L < sp::kMaxHDev; ++L) {
-            m.mb_level_off[L] = t.mb_level_off[S][L];
-            m.exp_off[L] = t.exp_off[S][L];
-            m.exp_n[L] = t.exp_n[S][L];
-            m.imp_full_n[L] = t.imp_full_n[S][L];
-            m.imp_phi_n[L] = t.imp_phi_n[S][L];
+            m.lists[L] = {t.imp_full_n[S][L], t.imp_phi_n[S][L], t.mb_level_off[S][L], 0};
+            m.exps[L] = {t.exp_off[S][L], t.exp_n[S][L]};
         }
+        if (m.exps[0].n != 0) return SP_EINVAL;
         for (size_t i = 0; i < t.same_succ[S].size(); ++i) m.same_succ[i] = t.same_succ[S][i];
     }
     for (int q = 0; q < 2; ++q)
@@ -592,10 +567,9 @@ int build_device_tables(sp_grid *g, int B)
     for (int S = 0; S < sp::kTypes; ++S)
         for (int L = 0; L < sp::kMaxHDev; ++L) {
             sp::TypeMeta &m = h.type[S];
-            m.imp_full_off[L] = (int)imp.size();
+            m.lists[L].imp_off = (int)imp.size();
             for (int i = 0; i < t.imp_full_n[S][L]; ++i)
                 imp.push_back((unsigned short)(t.imp_full[t.imp_full_off[S][L] + i] >> 16));  // (pi, c) index
-            m.imp_phi_off[L] = (int)imp.size();
             for (int i = 0; i < t.imp_phi_n[S][L]; ++i) imp.push_back((unsigned short)t.imp_phi[t.imp_phi_off[S][L] + i]);
         }
     while (imp.size() % 8) imp.push_back(0);
@@ -721,16 +695,18 @@ int choose_B(const sp_params &p, int requested)
 // Default workers of a base-8 region.  Many regions: 64, of which eight fit an
 // SM.  Where the widest phase (three region types) leaves an SM few regions at
 // a time, the chain of phases counts, and more workers shorten each region
-// (one simulation, 64 steps, us with 64 / 128 / 256 workers: 24^3 - / 431 / 401,
-// 32^3 564 / 432 / 433, 40^3 570 / 489 / 511, 48^3 654 / 535, 64^3 734 / 675,
-// 72^3 827 / 798, 80^3 934 / 985, 96^3 1255 / 1535).
+// (one simulation, 64 steps, us with 64 / 128 / 256 workers: 24^3 - / 346 / 273,
+// 32^3 - / 376 / 298, 40^3 - / 379 / 374, 48^3 - / 402, 64^3 577 / 556, 72^3 681 /
+// 686, 80^3 773 / 880, 96^3 1105 / 1390).
 int base8_threads(long long tiles, int sms) { return 2 * tiles <= sms ? 256 : tiles <= 5ll * sms ? 128 : 64; }
 
-// Default workers of a region of base B in a plan with the bases Bs.
+// Default workers of a region of base B in a plan with the bases Bs.  Base 16:
+// 480 (128^3, 128 steps, 320 / 384 / 480 / 512 / 768 workers: 3.40 / 3.37 / 3.32 /
+// 3.39 / 3.85 ms).
 int default_threads(const sp_grid *g, const std::vector<int> &Bs, int B)
 {
     if (B == 32) return sp::region_oct_workers();
-    if (B != 8) return B < 8 ? 64 : 384;
+    if (B != 8) return B < 8 ? 64 : 480;
     long long tiles = 0;  // regions of a type, of all simulations of this base
     for (int s = 0; s < g->n_sims; ++s)
         if (Bs[s] == B) tiles += (long long)(g->p[s].n[0] / B) * (g->p[s].n[1] / B) * (g->p[s].n[2] / B);

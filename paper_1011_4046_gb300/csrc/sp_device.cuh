@@ -13,28 +13,41 @@ namespace sp {
 // cell indices with shifts of at most 4 bits per axis).
 constexpr int kMaxHDev = 8;
 
+// What a level's step reads of the tables, in a few wide loads: the active box
+// (low corner, cells, its 2x2x2 blocks along x and z, and the multipliers for
+// quotients by c and a, see mdiv and block_cell) ...
+struct alignas(16) LevelBox {
+    int lo[3], cnt;
+    int a, c;
+    unsigned rc, ra;
+};
+// ... the imports landing at it (full and phi-only ones, offsets of their
+// mailbox chunk and of their lists, the phi-only list right after the full one)
+struct alignas(16) LevelLists {
+    int full_n, phi_n, mb_off, imp_off;
+};
+// ... and its exports.
+struct alignas(8) LevelExports {
+    int off, n;
+};
+
 // Per-type geometry and routing of one base size (one block per region type,
 // so a kernel can keep it in shared memory).
 struct alignas(16) TypeMeta {
     int levels, mb_size, n_same_succ, same_preds;
     int prev_preds;
     // band-base copy in units of (column, run of base_len cells along z):
-    // columns of the base box, 1/columns in FP32; the kernel chooses the run
-    // for its workers (base_len, and runs per column) in its own copy
+    // columns of the base box and the multiplier for quotients by them; the
+    // kernel chooses the run for its workers (base_len, and runs per column) in
+    // its own copy
     int base_cols;
-    float rcp_cols;
+    unsigned mul_cols;
     int base_len, base_runs;
-    Box3 active[kMaxHDev + 1];
     Box3 base_phi, base_pc;
-    // exact quotient decode (see fdiv below), reciprocals rounded to FP32:
-    // of each active box, 1/(w2/2) and 1/(w0/2) (its cells are taken in
-    // 2x2x2 blocks, see block_cell); of the base box, 1/w0 and 1/w1
-    float rcp_active[kMaxHDev + 1][2];
-    float rcp_base[2];
-    int imp_full_off[kMaxHDev], imp_full_n[kMaxHDev];
-    int imp_phi_off[kMaxHDev], imp_phi_n[kMaxHDev];
-    int mb_level_off[kMaxHDev];
-    int exp_off[kMaxHDev], exp_n[kMaxHDev];
+    unsigned mul_w0, pad_mul;  // for quotients by the base box's w0
+    LevelBox box[kMaxHDev + 1];
+    LevelLists lists[kMaxHDev];
+    LevelExports exps[kMaxHDev];
     Succ same_succ[kMaxSameSucc];
     // one mailbox slot: mailbox-reuse successors (in TablesDev::reuse) and
     // predecessors of a region of this type in a band after the first
@@ -471,6 +484,13 @@ __device__ __forceinline__ void red_release_cluster_add(unsigned raddr, int v)
 __device__ __forceinline__ void fence_acq_rel_gpu() { asm volatile("fence.acq_rel.gpu;" ::: "memory"); }
 
 #endif
+
+// floor(i / w) from the multiplier mdiv_mul(w), in one multiply and a shift where
+// fdiv's two conversions take ten times as long: i = w q + r with r < w, so
+// i mul / 2^20 lies in [q + r/w, q + r/w + i / 2^20], below q + 1 while i w < 2^20 (and the
+// product below 2^32); every range used is checked on the host.
+__host__ __device__ __forceinline__ unsigned mdiv_mul(int w) { return (1u << 20) / (unsigned)w + 1u; }
+__host__ __device__ __forceinline__ int mdiv(int i, unsigned mul) { return (int)(((unsigned)i * mul) >> 20); }
 
 // floor(i / w) for 0 <= i < 2^20 and 1 <= w <= 64, from rcp = 1/w rounded to
 // FP32: (i + 1/2) / w lies at least 1/(2w) away from an integer, and the two

@@ -142,19 +142,13 @@ static_assert(sizeof(SimDev) / 16 <= 32, "the manager warp copies a descriptor w
 
 // Export entries of a level are loaded into registers before the compute of
 // the next level (up to kExportPrefetch per worker thread); any remainder is
-// read in batches.  Three cover the average level of base 16 with 256
-// workers several times over; more cost registers and unrolled code for
-// entries that rarely exist.
-constexpr int kBaseRun = 4;  // most cells of a unit of the base copy
-constexpr int kExportPrefetch = 3;
+// read in batches.  Two cover the average level of base 16 with 256 workers;
+// more cost registers and unrolled code for entries that rarely exist
+// (128^3, base 16, 128 steps: 3.54 ms with one, 3.36 two, 3.41 three; base 8,
+// 64 steps: 2.75, 2.74, 2.79).
+constexpr int kExportPrefetch = 2;
 constexpr int kExportBatch = 4;
-// Per worker count: independent cell updates in flight per thread (measured:
-// one up to 128 workers, two for 256 and more; four were 3 % slower at base
-// 16), and the CTAs per SM the registers are budgeted for.  64 and 128 workers
-// serve base 8, whose small regions fit six and four CTAs per SM (an SM's
-// throughput grows almost linearly with the regions it holds); 256 and more
-// serve base 16, one CTA per SM.
-__host__ __device__ constexpr int region_cells_per_step(int nw) { return nw <= 128 ? 1 : 2; }
+constexpr int kBaseRun = 4;  // most cells of a unit of the base copy
 // Most threads of a CTA (workers and manager warps of its groups), which set the
 // register budget: eight regions of 64 workers, four of 128, one of more.
 __host__ __device__ constexpr int region_max_groups(int nw) { return nw <= 64 ? 8 : nw <= 128 ? 4 : 1; }
@@ -229,40 +223,24 @@ __device__ __forceinline__ void import_level(const float2 *__restrict__ mb, int 
         cp_async16(pc_s + pc_slot(c, lgB, B), mb + 2 * i);
         cp_async8(dst + pidx, mb + 2 * nf + i);
     }
-    for (int i = wt; i < np; i += NW) cp_async8(dst + pl[i], mb + 3 * nf + i);
+    for (int i = NW - 1 - wt; i < np; i += NW) cp_async8(dst + pl[i], mb + 3 * nf + i);
 }
 
 // The cells of level k are taken in 2x2x2 blocks (every extent of an active
 // box is even): linear index j -> block m = j >> 3, counted z fastest, then x,
-// then y (a = w0/2 and c = w2/2 blocks along x and z; rc = 1/c, ra = 1/a),
+// then y (a = w0/2 and c = w2/2 blocks along x and z),
 // and corner j & 7 of the block.  Eight consecutive threads then cover one
 // block: a block pair along z spans all sixteen 8-byte bank pairs of a phi
 // buffer (pitch B+2 = 2 mod 16 cells, plane pitch = 4 mod 16), and pc_slot
 // gives the block's eight (pi, c) pairs eight different bank groups.
-struct LevelBox {
-    Box3 A;
-    float rc, ra;
-    int a, c, cnt;
-    __device__ __forceinline__ void load(const TypeMeta &M, int k)
-    {
-        A = M.active[k];
-        rc = M.rcp_active[k][0];
-        ra = M.rcp_active[k][1];
-        const int w0 = A.hi[0] - A.lo[0], w2 = A.hi[2] - A.lo[2];
-        cnt = w0 * (A.hi[1] - A.lo[1]) * w2;
-        a = w0 >> 1;
-        c = w2 >> 1;
-    }
-};
-
 __device__ __forceinline__ void block_cell(int j, const LevelBox &L, int &ux, int &uy, int &uz)
 {
     const int m = j >> 3;
-    const int r = fdiv(m, L.rc);   // m / c
-    const int jj = fdiv(r, L.ra);  // r / a
-    ux = L.A.lo[0] + 2 * (r - jj * L.a) + (j & 1);
-    uy = L.A.lo[1] + 2 * jj + ((j >> 1) & 1);
-    uz = L.A.lo[2] + 2 * (m - r * L.c) + ((j >> 2) & 1);
+    const int r = mdiv(m, L.rc);   // m / c
+    const int jj = mdiv(r, L.ra);  // r / a
+    ux = L.lo[0] + 2 * (r - jj * L.a) + (j & 1);
+    uy = L.lo[1] + 2 * jj + ((j >> 1) & 1);
+    uz = L.lo[2] + 2 * (m - r * L.c) + ((j >> 2) & 1);
 }
 
 // Shared-memory slot of the (pi, c) pair of the cell at local u-coordinates.
@@ -272,54 +250,19 @@ __device__ __forceinline__ int pc_slot_of(int ux, int uy, int uz, int B)
     return (z * B + y) * B + (x ^ ((((y & 1) << 1) | ((z & 1) << 2)) & (B - 1)));
 }
 
-// Buffer and (pi, c) indices of U cells of level k, linear indices i, i +
-// stride, ... (see block_cell); past the end of the level they are unused.
-template <int U>
-__device__ __forceinline__ void cell_indices(int i, int stride, const LevelBox &L, int P, int B, int (&pidx)[U],
-                                             int (&cidx)[U])
+// Cell i of a level's box (see block_cell).
+__device__ __forceinline__ void evolve_cell(int i, const LevelBox &L, int P, int PP, int B, const float2 *__restrict__ prev_buf,
+                                            float2 *__restrict__ cur, float4 *__restrict__ pc_s, const LevelCoef &co,
+                                            const PhysConst &q)
 {
-#pragma unroll
-    for (int u = 0; u < U; ++u) {
-        int ux, uy, uz;
-        block_cell(i + u * stride, L, ux, uy, uz);
-        pidx[u] = (uz * P + uy) * P + ux;
-        cidx[u] = pc_slot_of(ux, uy, uz, B);
-    }
-}
-
-// U cells of level k: every input is loaded before any result is stored, so
-// the U updates are independent instruction streams (the compiler cannot prove
-// that a store to one cell's (pi, c) does not alias another cell's load).
-template <int U>
-__device__ __forceinline__ void evolve_cells(const int (&pidx)[U], const int (&cidx)[U], int P, int PP,
-                                             const float2 *__restrict__ prev_buf, float2 *__restrict__ cur,
-                                             float4 *__restrict__ pc_s, const LevelCoef &co, const PhysConst &q)
-{
-    float2 c[U], xm[U], xp[U], ym[U], yp[U], zm[U], zp[U];
-    float4 pc[U];
-#pragma unroll
-    for (int u = 0; u < U; ++u) {
-        const int p = pidx[u];
-        c[u] = prev_buf[p];
-        xm[u] = prev_buf[p - 1];
-        xp[u] = prev_buf[p + 1];
-        ym[u] = prev_buf[p - P];
-        yp[u] = prev_buf[p + P];
-        zm[u] = prev_buf[p - PP];
-        zp[u] = prev_buf[p + PP];
-        pc[u] = pc_s[cidx[u]];
-    }
-#pragma unroll
-    for (int u = 0; u < U; ++u) {
-        float2 pi = make_float2(pc[u].x, pc[u].y), cc = make_float2(pc[u].z, pc[u].w);
-        c[u] = site_update(c[u], xm[u], xp[u], ym[u], yp[u], zm[u], zp[u], pi, cc, co, q);
-        pc[u] = make_float4(pi.x, pi.y, cc.x, cc.y);
-    }
-#pragma unroll
-    for (int u = 0; u < U; ++u) {
-        cur[pidx[u]] = c[u];
-        pc_s[cidx[u]] = pc[u];
-    }
+    int ux, uy, uz;
+    block_cell(i, L, ux, uy, uz);
+    const int p = (uz * P + uy) * P + ux, c = pc_slot_of(ux, uy, uz, B);
+    const float4 v = pc_s[c];
+    float2 pi = make_float2(v.x, v.y), cc = make_float2(v.z, v.w);
+    cur[p] = site_update(prev_buf[p], prev_buf[p - 1], prev_buf[p + 1], prev_buf[p - P], prev_buf[p + P], prev_buf[p - PP],
+                         prev_buf[p + PP], pi, cc, co, q);
+    pc_s[c] = make_float4(pi.x, pi.y, cc.x, cc.y);
 }
 
 // The manager warp asks L2 for the next region's inputs while the worker is
@@ -669,14 +612,17 @@ __device__ void report_regions(const RegionArgs &a, int groups, const GroupSync 
 // A CTA hosts `groups` regions at a time, each a group of a manager warp and NW
 // workers with its own buffers and named barrier, which share the tables and
 // import lists (base 8: 10.8 KB beside 25.3 KB a region, so eight regions fit
-// an SM where six CTAs did).  Bound by latency, not by a pipe: at base 16 a
-// region takes 6.7 to 11 us, 0.8 us to request its base, 0.4 to wait for it and
-// 0.6 a level (import wait, barrier, index, update, export; 0.2 of it the
-// updates); 40 % of the issue slots and 28 % of DRAM are used (base 8: 62 and
-// 34 %).  On a small grid the hop from a region to its successor adds 2 us.
-// With the ready queue, and six CTAs at base 8, against this: 256^3, base 8, 8
-// steps 3.18 and 3.04 ms; 32^3, 64 steps 618 and 334 us; 192^3, base 16, 64
-// steps 6.35 and 6.13 ms; 64^3 540 and 425 us.
+// an SM where six CTAs did).  Bound by latency, not by a pipe: a
+// region is a chain of requesting its base (0.8 us at base 16), waiting for it
+// (0.4) and its levels (0.6 us each, imports, barrier, indices, update, exports),
+// in which every instruction counts: 40 % of the issue slots and 28 % of DRAM are
+// used (base 8: 62 and 34 %).  So the tables hold what a level reads in three wide
+// loads (128^3, base 16, 128 steps 3.60 to 3.50 ms), quotients are a multiply and
+// a shift (3.46), and a thread takes one cell at a time (two interleaved: 3.46,
+// one 3.41; the shorter code also leaves registers).  On a small grid the hop from
+// a region to its successor adds 2 us.  With the ready queue, and six CTAs at
+// base 8, against this: 256^3, base 8, 8 steps 3.18 and 2.85 ms; 32^3, 64 steps 618
+// and 300 us; 192^3, base 16, 64 steps 6.35 and 5.55 ms; 64^3 540 and 386 us.
 template <int NW, int BB>
 __global__ void __launch_bounds__(region_max_threads(NW), 1) region_kernel(RegionArgs a, int max_P_launch)
 {
@@ -755,6 +701,12 @@ __global__ void __launch_bounds__(region_max_threads(NW), 1) region_kernel(Regio
         return;
     }
     const int wt = tid - 32;  // worker thread index
+    // Its index with the warps in reverse, for the exports: the cells of a level and
+    // its full imports are dealt out from worker 0, the exports and the phi-only
+    // imports from the last one, so that no warp is last with all of them (128^3,
+    // base 16, 128 steps 3.71 ms with every list from worker 0, 3.60 so; 3.68 with
+    // each list starting where the one before ended).
+    const int wr = NW - 32 - (wt & ~31) + (wt & 31);
     for (int seq = 1;; ++seq) {
         if (wt == 0) {
             // bounded wait for the manager's handoff (a shared-memory poll: the
@@ -816,9 +768,9 @@ __global__ void __launch_bounds__(region_max_threads(NW), 1) region_kernel(Regio
             const int w0 = bp.hi[0] - bp.lo[0];
             const int ncol = M.base_cols, len = M.base_len, units = ncol * M.base_runs;
             for (int u = wt; u < units; u += NW) {
-                const int run = fdiv(u, M.rcp_cols);
+                const int run = mdiv(u, M.mul_cols);
                 const int i = u - run * ncol;
-                const int t1 = fdiv(i, M.rcp_base[0]);
+                const int t1 = mdiv(i, M.mul_w0);
                 const int ux = bp.lo[0] + i - t1 * w0;
                 const int uy = bp.lo[1] + t1;
                 const int oxy = (ux < bc.lo[0] || ux >= bc.hi[0]) + (uy < bc.lo[1] || uy >= bc.hi[1]);
@@ -845,10 +797,10 @@ __global__ void __launch_bounds__(region_max_threads(NW), 1) region_kernel(Regio
         const unsigned short *s_imp_t = s_imp + T.imp_smem;
         auto issue_level = [&](int L) {
             if (L <= H - 1) {
-                const int nf = M.imp_full_n[L], np = M.imp_phi_n[L];
-                if (nf + np > 0)
-                    import_level<NW>(mb_self + M.mb_level_off[L], nf, np, s_imp_t + M.imp_full_off[L],
-                                     s_imp_t + M.imp_phi_off[L], (L & 1) ? phi_buf1 : phi_buf0, pc_s, B, P, wt);
+                const LevelLists l = M.lists[L];
+                if (l.full_n + l.phi_n > 0)
+                    import_level<NW>(mb_self + l.mb_off, l.full_n, l.phi_n, s_imp_t + l.imp_off,
+                                     s_imp_t + l.imp_off + l.full_n, (L & 1) ? phi_buf1 : phi_buf0, pc_s, B, P, wt);
             }
             cp_async_commit();  // one group per level, empty or not
         };
@@ -862,47 +814,27 @@ __global__ void __launch_bounds__(region_max_threads(NW), 1) region_kernel(Regio
             float2 *__restrict__ cur = (k & 1) ? phi_buf1 : phi_buf0;
             issue_level(k + 1);  // lands in buffer (k+1) & 1 outside what level k reads
             // export entries of level k-1, loaded now, used after the compute
-            const int ne = k >= 2 ? M.exp_n[k - 1] : 0;
-            const int2 *el = T.exp + (k >= 2 ? M.exp_off[k - 1] : 0);
-            prefetch_entries<NW>(el, ne, pre, wt);
-            constexpr int U = region_cells_per_step(NW);
-            // bases 4 and 8: the level's box and the thread's next cells ahead of the
-            // barrier and of the updates (128^3, base 8: 5.79 ms, 6.03 without); at
-            // base 16 the registers they hold cost more than they hide (3.78, 3.72)
-            constexpr bool ahead = BB == 0;
-            int pidx[U], cidx[U];
-            LevelBox L;
-            if (ahead) {
-                L.load(M, k);
-                cell_indices<U>(wt, NW, L, P, B, pidx, cidx);
-            }
+            const LevelExports ex = M.exps[k - 1];  // none at level 0
+            const int ne = ex.n;
+            const int2 *el = T.exp + ex.off;
+            prefetch_entries<NW>(el, ne, pre, wr);
             cp_async_wait_pending(2);  // groups 0..k-1 (base, coefficients, levels < k) have landed
             named_barrier(kWorkerBarrier, NW);
-            // ---- evolve the cells of level k, several independent cells per step ----
+            // ---- evolve the cells of level k ----
             const LevelCoef co = s_coef[k - 1];
-            if (!ahead) L.load(M, k);
-            int i = wt;
-            for (; i + (U - 1) * NW < L.cnt; i += U * NW) {
-                if (!ahead) cell_indices<U>(i, NW, L, P, B, pidx, cidx);
-                evolve_cells<U>(pidx, cidx, P, PP, prev_buf, cur, pc_s, co, q);
-                if (ahead) cell_indices<U>(i + U * NW, NW, L, P, B, pidx, cidx);
-            }
-            for (; U > 1 && i < L.cnt; i += NW) {  // fewer than U left
-                int p1[1], c1[1];
-                cell_indices<1>(i, NW, L, P, B, p1, c1);
-                evolve_cells<1>(p1, c1, P, PP, prev_buf, cur, pc_s, co, q);
-            }
+            const LevelBox L = M.box[k];
+            for (int i = wt; i < L.cnt; i += NW) evolve_cell(i, L, P, PP, B, prev_buf, cur, pc_s, co, q);
             // ---- final surface of level k-1 (read-only data of level k-1) ----
-            if (ne > 0) export_entries<NW>(el, ne, pre, s_mb, prev_buf, pc_s, wt);
+            if (ne > 0) export_entries<NW>(el, ne, pre, s_mb, prev_buf, pc_s, wr);
         }
         const float2 *last = (nlev & 1) ? phi_buf1 : phi_buf0;
         if (nlev <= H - 1) {
             // ---- final surface of the last level ----
-            const int ne = M.exp_n[nlev];
-            const int2 *el = T.exp + M.exp_off[nlev];
-            prefetch_entries<NW>(el, ne, pre, wt);
+            const int ne = M.exps[nlev].n;
+            const int2 *el = T.exp + M.exps[nlev].off;
+            prefetch_entries<NW>(el, ne, pre, wr);
             named_barrier(kWorkerBarrier, NW);
-            export_entries<NW>(el, ne, pre, s_mb, last, pc_s, wt);
+            export_entries<NW>(el, ne, pre, s_mb, last, pc_s, wr);
         } else {
             named_barrier(kWorkerBarrier, NW);
             // ---- tops of the inverted pyramid: the next band's base ----

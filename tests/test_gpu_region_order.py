@@ -46,12 +46,12 @@ CASES = [
     ([((40, 32, 32), 2.0)], 8, 0, 128),  # 80
     ([((72, 72, 72), 2.0)], 8, 0, 128),  # 729, 128 workers up to 760
     ([((80, 80, 64), 2.0)], 8, 0, 64),  # 800: eight regions at a time on an SM
-    ([((32, 32, 32), 2.0)], 16, 0, 384),
+    ([((32, 32, 32), 2.0)], 16, 0, 480),
     ([((48, 32, 80), 0.0)], 16, 256, 256),
     ([((8, 12, 16), 2.0)], 4, 0, 64),
     ([((24, 16, 40), 2.0)], 4, 128, 128),
     ([((48, 16, 24), 2.0), ((16, 16, 16), 0.0), ((24, 56, 32), 1.0), ((16, 32, 24), 2.0)], 8, 0, 128),
-    ([((32, 64, 48), 1.0), ((32, 32, 32), 2.0), ((64, 48, 32), 0.0)], 16, 0, 384),
+    ([((32, 64, 48), 1.0), ((32, 32, 32), 2.0), ((64, 48, 32), 0.0)], 16, 0, 480),
 ]
 
 
