@@ -255,6 +255,9 @@ struct LatResident {
     __host__ __device__ size_t total(int groups) const { return region + groups * stride; }
 };
 
+// The next region of a group: none, its predecessors not all done, ready.
+enum { kLatNone, kLatWait, kLatReady };
+
 __device__ __forceinline__ int sext8(uint32_t w, int byte) { return (int)(w << (24 - 8 * byte)) >> 24; }
 
 // A CTA hosts several regions, each a group of NW threads with a barrier of its
@@ -265,7 +268,7 @@ __device__ __forceinline__ int sext8(uint32_t w, int byte) { return (int)(w << (
 // region), and a level waits for nothing but the barrier.  What bounds it at
 // edge 16 is the L1 data pipe (76 % busy, 43 wavefronts per 32 site-updates) and
 // the five regions that fit an SM: 1.384e11 site-updates/s at 240^3, 1.329e11
-// with the ring; 2, 3 or 2 interleaved cells a step 1.31, 1.30, 1.28e11; 160 or
+// with the ring (1.449e11 since a region follows the one before without a wait); 2, 3 or 2 interleaved cells a step 1.31, 1.30, 1.28e11; 160 or
 // 192 workers 1.35, 1.21e11.  Smaller regions gain most, as sharing the list
 // fits more of them: edge 12 0.785 to 1.05e11, edge 8 0.361 to 0.536e11.
 template <int NW>
@@ -274,7 +277,7 @@ __global__ void __launch_bounds__(lat_max_threads<NW>(), 1) lattice_kernel(const
     extern __shared__ __align__(16) unsigned char smem[];
     __shared__ int s_cell_off[4 * kLatMaxS + 1], s_cell_n[4 * kLatMaxS];
     __shared__ LatRegion s_regs[kLatMaxGroups];
-    __shared__ int s_stops[kLatMaxGroups];
+    __shared__ int s_stops[kLatMaxGroups], s_nexts[kLatMaxGroups];
     const int group = threadIdx.x / NW, tid = threadIdx.x - group * NW;
     const int R = 2 * a.s, W = 4 * a.s + 1, WW = W * W;
     const LatResident L(a.n_cell, a.n_slots, a.n_foot, W);
@@ -286,7 +289,7 @@ __global__ void __launch_bounds__(lat_max_threads<NW>(), 1) lattice_kernel(const
     char *const s_ph1 = reinterpret_cast<char *>(mine + L.ph1);
     unsigned *const s_yz = reinterpret_cast<unsigned *>(mine + L.yz);
     LatRegion &s_reg = s_regs[group];
-    volatile int &s_stop = s_stops[group];
+    volatile int &s_stop = s_stops[group], &s_next = s_nexts[group];
     for (int i = threadIdx.x; i < a.n_cell; i += blockDim.x) s_cell[i] = a.cell_wide[i];
     for (int i = threadIdx.x; i < WW; i += blockDim.x) s_row_x0[i] = a.row_x0[i];
     for (int i = threadIdx.x; i <= a.K; i += blockDim.x) {
@@ -295,28 +298,32 @@ __global__ void __launch_bounds__(lat_max_threads<NW>(), 1) lattice_kernel(const
     }
     // The control thread of a region is its last one: cells are dealt out from
     // thread 0, so it has the least evolution work at every level.  Its state:
-    // the next ticket, and early (relaxed) reads of the flags of the region
-    // that ticket names.
+    // the next ticket and the finished region whose flag is still to be set.  While
+    // a region's imports are on their way it sets that flag, decodes the region of
+    // the next ticket and, with three other threads of its warp, reads its
+    // predecessors' flags; if they are done, which is the rule once a layer has more
+    // regions than the GPU holds, the region follows without a wait, a fence or a
+    // barrier of its own (with a fence, the flag and the early reads' check between
+    // two regions: edge 16 1.390e11 site-updates/s at 240^3, now 1.449e11; edge 8
+    // 0.534 and 0.588e11; edge 20 1.121 and 1.205e11).
     const int ctl = NW - 1;
+    const bool ctl_warp = tid >= NW - 32;
     unsigned next = 0;
     int epoch = 0;
-    int fv[4] = {0, 0, 0, 0};
-    bool early = false;
+    int *unset = nullptr, unset_to = 0;  // flag of the finished region
     __syncthreads();  // the shared lists; a region waits only after it: another group of the CTA may hold its predecessor
     const int bar = 1 + group;
     if (tid == ctl) {
         epoch = *(volatile int *)&a.ctl->epoch;
         s_stop = 0;
         const unsigned t = atomicAdd(&a.ctl->head, 1u);
-        if (!lat_decode(a, t, epoch, &s_reg) || !lat_wait(a, s_reg))
-            s_stop = 1;
-        else
-            next = atomicAdd(&a.ctl->head, 1u);
+        if (!lat_decode(a, t, epoch, &s_reg) || !lat_wait(a, s_reg)) s_stop = 1;
     }
     named_barrier(bar, NW);
     const int ya = 8 * a.bank_a, zb = 8 * a.bank_b;  // byte steps of the residues
     while (!s_stop) {
         const LatRegion r = s_reg;
+        if (tid == ctl) next = atomicAdd(&a.ctl->head, 1u);
         const LatSimDev &sdr = a.sims[r.sim];
         const int n0 = sdr.n[0], cx = r.c[0] - R;
         // the first batch of import entries (their loads overlap the row set-up)
@@ -379,6 +386,21 @@ __global__ void __launch_bounds__(lat_max_threads<NW>(), 1) lattice_kernel(const
         }
         LevelCoef co = coef[r.tau_b + r.k_lo - 1];
         cp_async_commit();
+        if (ctl_warp) {
+            int more = 0;
+            if (tid == ctl) {
+                if (unset) st_release_gpu(unset, unset_to);
+                unset = nullptr;
+                more = lat_decode(a, next, epoch, &s_reg);  // every thread has copied the descriptor
+            }
+            __syncwarp();  // the descriptor
+            more = __shfl_sync(0xffffffffu, more, 31);
+            const int p = tid & 31;
+            bool ok = true;
+            if (more && p < 4 && s_reg.pred[p] >= 0) ok = ld_acquire_gpu(a.flags + s_reg.pred[p]) >= s_reg.Labs - 1;
+            ok = __all_sync(0xffffffffu, ok);
+            if (tid == ctl) s_next = !more ? kLatNone : ok ? kLatReady : kLatWait;
+        }
         cp_async_wait_all();
         named_barrier(bar, NW);
         for (int k = r.k_lo; k <= r.k_hi; ++k) {
@@ -387,14 +409,6 @@ __global__ void __launch_bounds__(lat_max_threads<NW>(), 1) lattice_kernel(const
             char *wr = odd ? s_ph1 : s_ph0;
             LevelCoef co_next = co;
             if (k < r.k_hi) co_next = coef[r.tau_b + k];
-            if (tid == ctl && k == r.k_lo) {
-                // every thread has copied the descriptor: decode the next
-                // region into it and read its predecessors' flags early
-                early = lat_decode(a, next, epoch, &s_reg);
-                if (early)
-                    for (int i = 0; i < 4; ++i)
-                        fv[i] = s_reg.pred[i] >= 0 ? ld_relaxed_gpu(a.flags + s_reg.pred[i]) : 0x7fffffff;
-            }
             float2 *gout = (par0 ^ odd) ? g_odd : g_even;
             const uint32_t exp_phi = k == r.k_hi ? ~0u : kLatWideExpPhi;  // the call's last level: export all
             const uint32_t exp_pc = k == r.k_hi ? ~0u : kLatWideExpPc;
@@ -429,20 +443,16 @@ __global__ void __launch_bounds__(lat_max_threads<NW>(), 1) lattice_kernel(const
                 a.trace[2 * r.id] = t_start;
                 a.trace[2 * r.id + 1] = globaltimer_ns();
             }
-            // One fence: release of this region's writes (made before the
-            // barrier above by every thread) to the flag store after it, and
-            // acquire for the early flag reads before it.
-            fence_acq_rel_gpu();
-            if (r.id != a.fault_drop) st_relaxed_gpu(a.flags + (size_t)((r.Labs & 3) * a.per_layer_all) + r.j, r.Labs);
-            if (!early) {
-                s_stop = 1;
-            } else {
-                const int need = s_reg.Labs - 1;
-                bool ready = true;
-                for (int i = 0; i < 4; ++i) ready = ready && fv[i] >= need;
-                if (!ready && !lat_wait(a, s_reg)) s_stop = 1;
-                if (!s_stop) next = atomicAdd(&a.ctl->head, 1u);
+            if (r.id != a.fault_drop) {
+                unset = a.flags + (size_t)((r.Labs & 3) * a.per_layer_all) + r.j;
+                unset_to = r.Labs;
             }
+        }
+        if (s_next == kLatReady) continue;
+        if (tid == ctl) {
+            if (unset) st_release_gpu(unset, unset_to);
+            unset = nullptr;
+            if (s_next == kLatNone || !lat_wait(a, s_reg)) s_stop = 1;
         }
         named_barrier(bar, NW);
     }
