@@ -66,12 +66,14 @@ SAMPLE_Z = 32
 # band-top state plus sloped faces, counted by brute force over one
 # steady-state band (each face cell written once, read by every consumer).
 ALG_BYTES_PER_UPDATE = {8: 42.8, 16: 25.3, 32: 13.8}
-MONO_BYTES_PER_UPDATE = 48.0
+# The whole-grid sweep takes two levels per pass over phi (8 B) and (pi, c)
+# (16 B), each read and written once.
+MONO_BYTES_PER_UPDATE = 24.0
 # On-chip (shared-memory) bytes per site-update of the region kernel: seven
 # phi reads (8 B) and one phi write, one (pi, c) read and write (16 B each).
 SMEM_BYTES_PER_UPDATE = 7 * 8 + 8 + 2 * 16
-# the lattice kernel also reads its cell entry (4 B) and row record (8 B)
-SMEM_BYTES_PER_UPDATE_LATTICE = SMEM_BYTES_PER_UPDATE + 4 + 8
+# the lattice kernel also reads its cell entry (8 B)
+SMEM_BYTES_PER_UPDATE_LATTICE = SMEM_BYTES_PER_UPDATE + 8
 # Shared-memory bandwidth of one GB300, nominal: 128 B per clock per SM (the
 # fallback when the measured peak is not available).
 SMS, SMEM_BYTES_PER_CLOCK = 152, 128

@@ -1,7 +1,8 @@
 // sp_kernels.cu -- sm_103a kernels of the region-scheduled leapfrog.
 //
-//   reset_kernel   arms the dependency counters and seeds the ready queue
-//   region_kernel  persistent: pops ready regions and evolves each on chip
+//   reset_kernel   arms the dependency counters and seeds the ready queue (learned
+//                  order and base 32; ticket_reset_kernel: a fixed order)
+//   region_kernel  persistent: takes regions in order and evolves each on chip
 //   sweep_kernel   monolithic whole-grid step (the comparator)
 //   feature_kernel inputs of the region cost model
 //
@@ -105,22 +106,23 @@ __global__ void seed_kernel(RegionArgs a)
 }
 
 // ------------------------------------------------------------ region kernel
-// Warp-specialised persistent kernel.  Warp 0 is the manager (the paper's
-// manager process, Sec. 4); the other NW threads are the worker that
-// evolves one region at a time.
+// Warp-specialised persistent kernel.  A group is a manager warp (the paper's
+// manager process, Sec. 4) and the NW threads of a worker that evolves one
+// region at a time; a CTA holds one group or several (region_kernel, below).
 //
-// Manager: while the workers evolve region R it waits (bounded) for the next
-// queue position to be filled.  As soon as the workers report R done it hands
-// them the next region and only then releases R's successors (GPU-scope fence,
-// acq_rel decrements, push at zero), so the release overlaps the next
-// region's work.  If the next region is not ready it releases R first (the
-// next region may be one of R's successors).
+// Manager, fixed order: manager_tickets.  With the learned order (manager_loop),
+// while the workers evolve region R it waits (bounded) for the next queue
+// position to be filled.  As soon as the workers report R done it hands them the
+// next region and only then releases R's successors (GPU-scope fence, acq_rel
+// decrements, push at zero), so the release overlaps the next region's work.
+// If the next region is not ready it releases R first (the next region may be
+// one of R's successors).
 //
-// Worker shared memory, in order: two phi buffers (levels of alternating
+// Shared memory of a group: two phi buffers (levels of alternating
 // parity) of (B+2)^3 float2 for the region box plus its halo; one float4
-// (pi, c) per own cell (B^3, slots permuted by pc_slot); the launch's tables
-// (geometry and routing per region type); the band's level coefficients; the
-// import lists.  The tables and import lists are copied once per launch and
+// (pi, c) per own cell (B^3, slots permuted by pc_slot); the band's level
+// coefficients.  Of the CTA: the launch's tables (geometry and routing per
+// region type) and import lists.  The tables and import lists are copied once per launch and
 // the simulation descriptor travels with the handoff, so no step of a region
 // waits on a table read from global memory (export entries are read through
 // L1, one level ahead).
@@ -270,8 +272,8 @@ __device__ __forceinline__ void evolve_cell(int i, const LevelBox &L, int P, int
 // arrays, one request per 128-byte line) and the region's whole mailbox (all
 // levels; the region is ready, so every chunk is written).  Prefetches of
 // addresses inside the arrays never fault and change no data.  Used at base
-// 16 (one region per SM: 7.95 -> 7.56 ms at 128^3); at base 8, with six CTAs
-// per SM prefetching, it measured 10 % slower.
+// 16 (one region per SM: 192^3, 64 steps 6.57 ms without, 6.20 with it); at base
+// 8, with several regions per SM prefetching, it measured 10 % slower.
 __device__ void prefetch_region_l2(const SimDev &sd, const TypeMeta &M, const RegionInfo &r, int lane)
 {
     const int B = sd.B, H = sd.H;
