@@ -1263,7 +1263,15 @@ int plan_lattice(sp_grid *g, const std::vector<int> &Bs, int threads)
         // site-updates/s at s = 3, 0.80e11 with 128), 128 at s = 4 (1.384e11; 64:
         // 0.91e11, 192: 1.21e11), 256 at s = 5, 512 at s = 6
         const int s_lat = it->first;
-        c.threads = threads ? threads : s_lat <= 3 ? 64 : s_lat <= 4 ? 128 : s_lat == 5 ? 256 : 512;
+        // Edges 8 and 12 take 64 workers where a layer has regions for every SM's
+        // places, 128 where the chain of layers counts (M^3 positions, 100 steps, us
+        // with 64 / 128: edge 12, M = 6 744 / 564, 8 996 / 1085; edge 8 642 / 543,
+        // 743 / 918).
+        long long layer_regions = 0;
+        for (int s = 0; s < g->n_sims; ++s)
+            layer_regions += 4ll * (g->p[s].n[0] / (4 * s_lat)) * (g->p[s].n[1] / (4 * s_lat)) * (g->p[s].n[2] / (4 * s_lat));
+        const bool few = s_lat >= 2 && layer_regions <= 7ll * g->sm_count;
+        c.threads = threads ? threads : s_lat <= 3 && !few ? 64 : s_lat <= 4 ? 128 : s_lat == 5 ? 256 : 512;
         sp::LatConfig lc;
         e = sp::lattice_config(t, c.threads, &lc);
         if (e != cudaSuccess || lc.ctas_per_sm < 1) return SP_EINVAL;
