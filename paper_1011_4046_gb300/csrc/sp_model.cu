@@ -696,6 +696,14 @@ void epoch_order(uint64_t seed, int ep, int64_t n, std::vector<int> *order)
     }
 }
 
+// Waits for a stream on the way out of a call, so that host values its queued
+// copies still read outlive them whichever way the call ends (declared after
+// those values).
+struct Drain {
+    cudaStream_t stream;
+    ~Drain() { cudaStreamSynchronize(stream); }
+};
+
 double uniform01(uint64_t seed, uint64_t i) { return (double)(splitmix64(seed, i) >> 11) * 0x1.0p-53; }
 
 }  // namespace
@@ -894,7 +902,13 @@ int sp_model_train(sp_model *m, const float *x_dev, const float *y_dev, int64_t 
     if (grow_buf(&m->order, &m->cap_order, total) != cudaSuccess) return SP_ENOMEM;
     if (grow_buf(&m->losses, &m->cap_losses, steps) != cudaSuccess) return SP_ENOMEM;
     const float beta1 = 0.9f, beta2 = 0.999f, eps = 1e-8f;
+    // What the call's copies read or write on the host.  An asynchronous copy from
+    // pageable memory may read it as late as its turn on the stream, behind the
+    // training before it, so every epoch's order stands by itself.
     std::vector<float2> corr(steps);
+    std::vector<std::vector<int>> orders(order_host ? 0 : (size_t)epochs);
+    std::vector<float> pred((size_t)n);
+    const Drain drain{m->stream};
     for (size_t k = 0; k < steps; ++k) {
         const double t = (double)(m->adam_t + (int64_t)k + 1);
         corr[k] = make_float2((float)(1.0 / (1.0 - std::pow((double)beta1, t))), (float)(1.0 / (1.0 - std::pow((double)beta2, t))));
@@ -908,13 +922,12 @@ int sp_model_train(sp_model *m, const float *x_dev, const float *y_dev, int64_t 
         if (e != cudaSuccess) return SP_ECUDA;
     }
     // epoch by epoch: while the GPU trains one, the host makes the next one's order
-    std::vector<int> order;
     size_t step = 0;
     for (int ep = 0; ep < epochs; ++ep) {
         const int *src = order_host ? order_host + (size_t)ep * n : nullptr;
         if (!src) {
-            epoch_order(order_seed, ep, n, &order);
-            src = order.data();
+            epoch_order(order_seed, ep, n, &orders[(size_t)ep]);
+            src = orders[(size_t)ep].data();
         }
         int *const d_order = m->order + (size_t)ep * n;
         e = cudaMemcpyAsync(d_order, src, (size_t)n * sizeof(int), cudaMemcpyHostToDevice, m->stream);
@@ -947,7 +960,6 @@ int sp_model_train(sp_model *m, const float *x_dev, const float *y_dev, int64_t 
     }
     // bucket thresholds: quartiles of the trained network's predictions on the
     // training set (order statistics, largest first)
-    std::vector<float> pred((size_t)n);
     if (grow_buf(&m->pred, &m->cap_pred, (size_t)n) != cudaSuccess) return SP_ENOMEM;
     e = infer<false>(m->theta, nullptr, x_dev, n, m->pred, nullptr, m->sms, m->stream);
     if (e == cudaSuccess) e = cudaMemcpyAsync(pred.data(), m->pred, (size_t)n * sizeof(float), cudaMemcpyDeviceToHost, m->stream);
