@@ -332,7 +332,10 @@ __global__ void adam_kernel(float *__restrict__ theta, float *__restrict__ m, fl
 // tiles over the samples.
 constexpr int kTrainThreads = 256;
 constexpr int kTrainChunk = 16;  // samples of a pass
-constexpr int kTrainCtas = 16;   // most CTAs of the cluster (8 where 16 do not fit)
+#ifndef SP_TRAIN_CTAS  // a test builds the kernel of 8
+#define SP_TRAIN_CTAS 16
+#endif
+constexpr int kTrainCtas = SP_TRAIN_CTAS;  // most CTAs of the cluster (8 where 16 do not fit)
 // Largest minibatch of this path (4096 samples: 59 us a step, 76 as launches
 // over many SMs, which take 8192 in 83)
 constexpr int kTrainMaxBatch = 4096;
@@ -638,11 +641,13 @@ cudaError_t train_launch_t(const TrainArgs &a, cudaStream_t st, bool probe)
     return e != cudaSuccess ? e : clusters > 0 ? cudaSuccess : cudaErrorInvalidConfiguration;
 }
 
-// CTAs of the training cluster on the current device, 0: none fits.
+// CTAs of the training cluster on the current device, 0: none fits.  A size that
+// does not fit is an answer, not an error of the call: it is cleared.
 int train_ctas()
 {
     const TrainArgs none = {};
     if (train_launch_t<kTrainCtas>(none, nullptr, true) == cudaSuccess) return kTrainCtas;
+    cudaGetLastError();
     if (train_launch_t<8>(none, nullptr, true) == cudaSuccess) return 8;
     cudaGetLastError();
     return 0;

@@ -25,7 +25,7 @@ struct Op {
 
 size_t g_capacity, g_used, g_peak;
 bool g_deferred;
-unsigned g_refused_cluster;  // cluster size whose occupancy query fails
+unsigned g_refused_cluster;  // occupancy queries of clusters this large fail (0: none)
 cudaError_t g_last;
 std::map<void *, size_t> g_mem;
 std::vector<Op> g_ops, g_done;
@@ -167,7 +167,8 @@ cudaError_t cudaOccupancyMaxActiveBlocksPerMultiprocessorWithFlags(int *n, const
 cudaError_t cudaOccupancyMaxActiveClusters(int *n, const void *, const cudaLaunchConfig_t *c)
 {
     for (unsigned i = 0; i < c->numAttrs; ++i)
-        if (c->attrs[i].id == cudaLaunchAttributeClusterDimension && c->attrs[i].val.clusterDim.x == g_refused_cluster)
+        if (c->attrs[i].id == cudaLaunchAttributeClusterDimension && g_refused_cluster &&
+            c->attrs[i].val.clusterDim.x >= g_refused_cluster)
             return *n = 0, result(cudaErrorInvalidValue);
     return *n = 4, cudaSuccess;
 }
