@@ -243,8 +243,12 @@ int sp_region_plan(sp_grid *g, int32_t base_B, int32_t block_shape, int32_t orde
  * distinct base (largest base first, each launch sized for its base); a
  * remainder of fewer than B/2 steps runs as whole-grid steps with the same
  * arithmetic.  SP_MONOLITHIC runs every step as a whole-grid sweep (bit-exact
- * with the region path).  Unless SP_ASYNC is given the call synchronises the
- * stream and reports device errors.
+ * with the region path); where there is memory to spare, sweeps of four or more
+ * steps of a large grid take 16 more bytes per site, which the handle keeps up
+ * to a sixteenth of the device memory (more: until the next synchronous call
+ * ends) and gives back before a plan or when an allocation of its own fails.
+ * Unless SP_ASYNC is given the call synchronises the stream and reports device
+ * errors.
  * Errors: SP_EINVAL, SP_ENOTPLANNED, SP_EUNSTABLE (dt^2 (12/dx^2 + 2 lambda
  * eta^2 a^2) >= 4 at some level), SP_ETIMEOUT, SP_ECUDA.
  */

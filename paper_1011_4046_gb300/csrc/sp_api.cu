@@ -223,8 +223,9 @@ struct sp_grid {
     size_t cap_trace = 0;
     float2 *d_tmp = nullptr;
     size_t cap_tmp = 0;
-    float4 *d_tmp_pc = nullptr;  // two-level sweep passes only
+    float4 *d_tmp_pc = nullptr;  // two-level sweep passes only (release_sweep_copy)
     size_t cap_tmp_pc = 0;
+    bool keep_tmp_pc = false;    // beyond a synchronous call
     char *d_epart = nullptr;  // diagnostics: sums per block, and the result
     size_t cap_epart = 0;
     sp::DiagOut *d_diag = nullptr;
@@ -262,6 +263,33 @@ struct sp_grid {
 };
 
 namespace {
+
+// Gives back the second (pi, c) copy of two-level sweep passes, which only makes
+// sweeps faster: whatever else needs the memory goes before it.
+void release_sweep_copy(sp_grid *g)
+{
+    if (!g->d_tmp_pc) return;
+    if (g->sweep_graph.exec && g->sweep_graph.tmp_pc) {
+        cudaGraphExecDestroy(g->sweep_graph.exec);
+        g->sweep_graph = SweepGraph();
+    }
+    cudaFree(g->d_tmp_pc);
+    g->d_tmp_pc = nullptr;
+    g->cap_tmp_pc = 0;
+}
+
+// grow() for what a call cannot do without.
+template <class T>
+cudaError_t grow_needed(sp_grid *g, T **p, size_t *cap, size_t need)
+{
+    cudaError_t e = grow(p, cap, need);
+    if (e == cudaErrorMemoryAllocation && g->d_tmp_pc) {
+        cudaGetLastError();
+        release_sweep_copy(g);
+        e = grow(p, cap, need);
+    }
+    return e;
+}
 
 int cuda_err(cudaError_t e) { return e == cudaSuccess ? SP_OK : SP_ECUDA; }
 
@@ -761,7 +789,10 @@ int enqueue_sweep(sp_grid *g, int s, int64_t nsteps, int64_t first_local, const 
 // (32 B a site) no longer sit in L2 (measured per level, one at a time / two:
 // 96^3 6.3 / 7.6 us, 128^3 11.4 / 13.2, 144^3 22.5 / 17.1, 160^3 35.2 / 20.9,
 // 256^3 133 / 71, 400^3 509 / 257; 2.5e6 sites are 80 MB), and where the
-// second copy of (pi, c) leaves a sixteenth of the device memory free.
+// second copy of (pi, c) leaves a sixteenth of the device memory free.  The copy
+// is kept up to a sixteenth of the device memory; a larger one is given back at
+// the end of a synchronous call (1280^3, 33.6 GB: 12 ms to take and give back, a
+// step 9.3 ms against 16.5), any one before a plan or when memory runs out.
 bool sweep_by_pairs(sp_grid *g, int s, int64_t nsteps)
 {
     const size_t sites = (size_t)sites_of(g->p[s]);
@@ -771,6 +802,7 @@ bool sweep_by_pairs(sp_grid *g, int s, int64_t nsteps)
     if (cudaMemGetInfo(&free_b, &total_b) != cudaSuccess) return false;
     free_b += g->cap_tmp_pc * sizeof(float4);  // grow() frees the smaller copy first
     if (free_b < sites * sizeof(float4) + total_b / 16) return false;
+    g->keep_tmp_pc = sites * sizeof(float4) <= total_b / 16;
     if (grow(&g->d_tmp_pc, &g->cap_tmp_pc, sites) == cudaSuccess) return true;
     cudaGetLastError();  // the one-level path needs no such copy
     return false;
@@ -784,10 +816,10 @@ int sweep_steps(sp_grid *g, int s, int64_t nsteps, int64_t first_local, const sp
 {
     if (nsteps <= 0) return SP_OK;
     const int64_t sites = sites_of(g->p[s]);
-    cudaError_t e = grow(&g->d_tmp, &g->cap_tmp, (size_t)sites);
+    cudaError_t e = grow_needed(g, &g->d_tmp, &g->cap_tmp, (size_t)sites);
     if (e != cudaSuccess) return SP_ENOMEM;
     const bool pairs = sweep_by_pairs(g, s, nsteps);
-    if (g->stream == nullptr) return enqueue_sweep(g, s, nsteps, first_local, d_coef_sim, pairs);
+    if (g->stream == nullptr || (pairs && !g->keep_tmp_pc)) return enqueue_sweep(g, s, nsteps, first_local, d_coef_sim, pairs);
     SweepGraph &sg = g->sweep_graph;
     if (!(sg.exec && sg.sim == s && sg.steps == nsteps && sg.first_local == first_local && sg.coef == d_coef_sim &&
           sg.phi == g->phi[s] && sg.tmp == g->d_tmp && sg.tmp_pc == (pairs ? g->d_tmp_pc : nullptr))) {
@@ -1072,8 +1104,8 @@ int evolve_lattice(sp_grid *g, int64_t n_steps, bool trace, bool timing)
         sim_off.push_back(first);
         launches.push_back(l);
     }
-    cudaError_t e = grow(&g->d_lsims, &g->cap_lsims, sims.size());
-    if (e == cudaSuccess && trace) e = grow(&g->d_trace, &g->cap_trace, 2 * (size_t)trace_total);
+    cudaError_t e = grow_needed(g, &g->d_lsims, &g->cap_lsims, sims.size());
+    if (e == cudaSuccess && trace) e = grow_needed(g, &g->d_trace, &g->cap_trace, 2 * (size_t)trace_total);
     if (e != cudaSuccess) return SP_ENOMEM;
     for (size_t i = 0; i < launches.size(); ++i) {
         launches[i].a.sims = g->d_lsims + sim_off[i];
@@ -1585,6 +1617,7 @@ int sp_grid_create(const sp_params *p, int32_t n_sims, void *const *state_dev, v
 int sp_region_plan(sp_grid *g, int32_t base_B, int32_t block_shape, int32_t order, const char *model_path)
 {
     if (!g) return SP_EINVAL;
+    release_sweep_copy(g);
     if (g->shape_opt == SP_SHAPE_LATTICE) {
         // congruent regions in a fixed topological (layer) order: nothing to learn
         if (order != SP_ORDER_STATIC) return SP_EINVAL;
@@ -1649,7 +1682,7 @@ int sp_evolve(sp_grid *g, int64_t n_steps, uint32_t flags)
     cudaError_t e = cudaSuccess;
     if (coef.size() != g->up_coef.size() ||
         std::memcmp(coef.data(), g->up_coef.data(), coef.size() * sizeof(sp::LevelCoef)) != 0) {
-        e = grow(&g->d_coef, &g->cap_coef, coef.size());
+        e = grow_needed(g, &g->d_coef, &g->cap_coef, coef.size());
         if (e != cudaSuccess) return SP_ENOMEM;
         e = cudaMemcpyAsync(g->d_coef, coef.data(), coef.size() * sizeof(sp::LevelCoef), cudaMemcpyHostToDevice,
                             g->stream);
@@ -1751,17 +1784,17 @@ int sp_evolve(sp_grid *g, int64_t n_steps, uint32_t flags)
                 max_flags = std::max(max_flags, total);
         }
         if (!launches.empty()) {
-            e = grow(&g->d_sims, &g->cap_sims, sims.size());
-            if (e == cudaSuccess) e = grow(&g->d_counters, &g->cap_counters, max_total);
-            if (e == cudaSuccess) e = grow(&g->d_queue, &g->cap_queue, max_total);
+            e = grow_needed(g, &g->d_sims, &g->cap_sims, sims.size());
+            if (e == cudaSuccess) e = grow_needed(g, &g->d_counters, &g->cap_counters, max_total);
+            if (e == cudaSuccess) e = grow_needed(g, &g->d_queue, &g->cap_queue, max_total);
             if (e == cudaSuccess && max_flags && g->cap_flags < (size_t)max_flags + 1) {
-                e = grow(&g->d_flags, &g->cap_flags, (size_t)max_flags + 1);
+                e = grow_needed(g, &g->d_flags, &g->cap_flags, (size_t)max_flags + 1);
                 if (e == cudaSuccess) e = cudaMemsetAsync(g->d_flags, 0, g->cap_flags * sizeof(int), g->stream);
             }
-            if (e == cudaSuccess && trace) e = grow(&g->d_trace, &g->cap_trace, 2 * (size_t)all_total);
-            if (e == cudaSuccess && feats) e = grow(&g->d_feat, &g->cap_feat, (size_t)SP_MODEL_FEATURES * all_total);
-            if (e == cudaSuccess && feats) e = grow(&g->d_simf, &g->cap_simf, sims.size());
-            if (e == cudaSuccess && learned) e = grow(&g->d_prio, &g->cap_prio, (size_t)all_total);
+            if (e == cudaSuccess && trace) e = grow_needed(g, &g->d_trace, &g->cap_trace, 2 * (size_t)all_total);
+            if (e == cudaSuccess && feats) e = grow_needed(g, &g->d_feat, &g->cap_feat, (size_t)SP_MODEL_FEATURES * all_total);
+            if (e == cudaSuccess && feats) e = grow_needed(g, &g->d_simf, &g->cap_simf, sims.size());
+            if (e == cudaSuccess && learned) e = grow_needed(g, &g->d_prio, &g->cap_prio, (size_t)all_total);
             if (e != cudaSuccess) return SP_ENOMEM;
             for (GroupLaunch &gl : launches) {  // device addresses, now that the buffers exist
                 gl.a.sims = g->d_sims + gl.sim_off;
@@ -1811,7 +1844,7 @@ int sp_evolve(sp_grid *g, int64_t n_steps, uint32_t flags)
             const int H = g->B[s] / 2;
             const int64_t done = (n_steps / H) * H;
             if (n_steps - done > 0) {
-                e = grow(&g->d_tmp, &g->cap_tmp, (size_t)sites_of(g->p[s]));
+                e = grow_needed(g, &g->d_tmp, &g->cap_tmp, (size_t)sites_of(g->p[s]));
                 if (e != cudaSuccess) return SP_ENOMEM;
             }
         }
@@ -1828,6 +1861,7 @@ int sp_evolve(sp_grid *g, int64_t n_steps, uint32_t flags)
     if (flags & SP_ASYNC) return SP_OK;
     e = cudaStreamSynchronize(g->stream);
     if (e != cudaSuccess) return SP_ECUDA;
+    if (!g->keep_tmp_pc) release_sweep_copy(g);
     if (!mono) return collect_device_error(g);
     return SP_OK;
 }
@@ -1915,7 +1949,7 @@ int sp_read_surface(const sp_grid *gc, int32_t sim, int32_t what, void *dst, siz
         if (dst_is_device) {
             w = (signed char *)dst;
         } else {
-            e = grow(&g->d_wind, &g->cap_wind, (size_t)(3 * sites));
+            e = grow_needed(g, &g->d_wind, &g->cap_wind, (size_t)(3 * sites));
             if (e != cudaSuccess) return SP_ENOMEM;
             w = g->d_wind;
         }
@@ -1927,7 +1961,7 @@ int sp_read_surface(const sp_grid *gc, int32_t sim, int32_t what, void *dst, siz
     }
     case SP_SURF_DIAG: {
         if (dst_bytes < sizeof(sp_diag)) return SP_EINVAL;
-        e = grow(&g->d_epart, &g->cap_epart, sp::diag_scratch_bytes(p.n));
+        e = grow_needed(g, &g->d_epart, &g->cap_epart, sp::diag_scratch_bytes(p.n));
         if (e != cudaSuccess) return SP_ENOMEM;
         double tau, a, d;
         level_physics(p, g->level[sim], &tau, &a, &d);
