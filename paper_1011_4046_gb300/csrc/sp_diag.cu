@@ -233,6 +233,9 @@ __global__ void __launch_bounds__(kDiagThreads, 3) diag_kernel(const DiagArgs a)
         }
         if (ENERGY) {
             const float ks = kin.s.x + kin.s.y, gs = grad.s.x + grad.s.y;
+            // without a vacuum value |phi|^2 can fall below the FP32 range and leave
+            // m = 0 where phi is not: a zero sum then says nothing
+            if (a.eta2 == 0.0) pot_bits = 1u;
             slow = !(a.fast && in_range(ks, kin.e.x + kin.e.y, kin_bits) &&
                      in_range(gs, grad.e.x + grad.e.y, grad_bits) && in_range(ps, pe, pot_bits));
             if (slow) column_fp64(a, oa, ob, od, z0, z1, en);
