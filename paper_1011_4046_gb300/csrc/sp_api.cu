@@ -785,10 +785,9 @@ int enqueue_sweep(sp_grid *g, int s, int64_t nsteps, int64_t first_local, const 
 }
 
 // Whether the steps of a sweep call go two levels at a time: from four steps
-// on (fewer hold no even number of pairs), where the state and its phi copy
-// (32 B a site) no longer sit in L2 (measured per level, one at a time / two:
-// 96^3 6.3 / 7.6 us, 128^3 11.4 / 13.2, 144^3 22.5 / 17.1, 160^3 35.2 / 20.9,
-// 256^3 133 / 71, 400^3 509 / 257; 2.5e6 sites are 80 MB), and where the
+// on (fewer hold no even number of pairs), where that is faster for the grid's
+// shape (columns_pay; per level, one at a time / two: 144^3 22.5 / 17.1 us, 160^3
+// 35.2 / 20.9, 256^3 133 / 71, 400^3 509 / 257), and where the
 // second copy of (pi, c) leaves a sixteenth of the device memory free.  The copy
 // is kept up to a sixteenth of the device memory; a larger one is given back at
 // the end of a synchronous call (1280^3, 33.6 GB: 12 ms to take and give back, a
@@ -796,7 +795,7 @@ int enqueue_sweep(sp_grid *g, int s, int64_t nsteps, int64_t first_local, const 
 bool sweep_by_pairs(sp_grid *g, int s, int64_t nsteps)
 {
     const size_t sites = (size_t)sites_of(g->p[s]);
-    if (nsteps < 4 || sites < 2500000) return false;
+    if (nsteps < 4 || !sp::columns_pay(g->phi[s], g->pc[s], g->p[s].n, g->sm_count)) return false;
     if (g->d_tmp_pc && g->cap_tmp_pc >= sites) return true;
     size_t free_b = 0, total_b = 0;
     if (cudaMemGetInfo(&free_b, &total_b) != cudaSuccess) return false;

@@ -254,30 +254,68 @@ __global__ void __launch_bounds__(32 * kColWarps, 1) column_kernel(const ColArgs
 
 }  // namespace
 
+namespace {
+
+// Tiles (of even width, evenly cut) and chunks of planes for a grid.  A chunk
+// takes 2 x halo steps more than its planes, and the SMs take the chunks in
+// waves; the fewest steps over all waves wins.  Returns those steps.
+long long plan_columns(const int n[3], int sm_count, ColArgs *a)
+{
+    const int tx = (n[0] + kColX - 1) / kColX, ty = (n[1] + kColY - 1) / kColY;
+    a->vx = ((n[0] + tx - 1) / tx + 1) & ~1;
+    a->vy = (n[1] + ty - 1) / ty;
+    const long long tiles = (long long)((n[0] + a->vx - 1) / a->vx) * ((n[1] + a->vy - 1) / a->vy);
+    long long best = 0;
+    for (int chunks = 1; chunks <= n[2]; ++chunks) {
+        const int zc = (n[2] + chunks - 1) / chunks;
+        const long long ctas = tiles * ((n[2] + zc - 1) / zc);
+        const long long steps = ((ctas + sm_count - 1) / sm_count) * (zc + 2 * kColHalo);
+        if (best == 0 || steps < best) best = steps, a->zc = zc;
+        if (ctas > 32ll * sm_count) break;
+    }
+    return best;
+}
+
+// Whether a lane's two sites are one aligned pair of phi and of (pi, c).
+bool columns_vec(int nx, const void *phi_a, const void *phi_b, const void *pc_a, const void *pc_b)
+{
+    return (nx & 1) == 0 && (((uintptr_t)phi_a | (uintptr_t)phi_b) & 15) == 0 && (((uintptr_t)pc_a | (uintptr_t)pc_b) & 31) == 0;
+}
+
+}  // namespace
+
+// Whether a pass of two levels beats two one-level sweeps.  The pass takes its
+// steps over all waves times 1.5 us (1.8 where the rows are no aligned pairs),
+// whatever part of a tile the grid fills: a thin grid, one just over a tile's
+// width or one of few planes pays for whole tiles and halos (1024 x 4 x 1024: 185
+// us, two levels one at a time 68; 20 x 512 x 512: 122 and 99; 137^3: 39 and 33).
+// The one-level sweep takes 16 us per 1e6 sites for two levels beyond L2, 11.5
+// where part of the state and its phi copy (32 B a site) still hits it, up to half
+// as much again where lanes of its 32-wide blocks stay idle, and always wins where
+// all of the state hits (128^3: 11.4 us a level against 13.2).  Over 249 grids of
+// 2.5e6 to 1e8 sites, sides 4 to 16384, the side it takes is within 2 % of the
+// better one (level pairs beyond 2.5e6 sites, whatever the shape: up to 2.7 times
+// slower).
+bool columns_pay(const float2 *phi, const float4 *pc, const int n[3], int sm_count)
+{
+    const double sites = (double)n[0] * n[1] * n[2];
+    if (sites < 2500000.0) return false;
+    ColArgs a = {};
+    const double pass = (double)plan_columns(n, sm_count, &a) * (columns_vec(n[0], phi, nullptr, pc, nullptr) ? 1.5 : 1.8);
+    const double idle = 1.0 - n[0] / (32.0 * ((n[0] + 31) / 32));
+    return pass <= 1e-6 * sites * (sites < 2800000.0 ? 11.5 : 16.0) * (1.0 + 0.5 * idle);
+}
+
 cudaError_t launch_columns(const float2 *phi_in, const float4 *pc_in, float2 *phi_out, float4 *pc_out, const int n[3],
                            const LevelCoef *coef, PhysConst q, int sm_count, cudaStream_t st)
 {
     ColArgs a{phi_in, pc_in, phi_out, pc_out, coef, q, n[0], n[1], n[2], 0, 0, 0, 0};
-    // tiles of even width, evenly cut
-    const int tx = (n[0] + kColX - 1) / kColX, ty = (n[1] + kColY - 1) / kColY;
-    a.vx = ((n[0] + tx - 1) / tx + 1) & ~1;
-    a.vy = (n[1] + ty - 1) / ty;
-    const int gx = (n[0] + a.vx - 1) / a.vx, gy = (n[1] + a.vy - 1) / a.vy;
-    // chunks of planes: a chunk takes 2 x halo steps more than its planes, and
-    // the SMs take the chunks in waves; the fewest steps over all waves wins
-    long long best = 0;
-    for (int chunks = 1; chunks <= n[2]; ++chunks) {
-        const int zc = (n[2] + chunks - 1) / chunks;
-        const long long ctas = (long long)gx * gy * ((n[2] + zc - 1) / zc);
-        const long long steps = ((ctas + sm_count - 1) / sm_count) * (zc + 2 * kColHalo);
-        if (best == 0 || steps < best) best = steps, a.zc = zc;
-        if (ctas > 32ll * sm_count) break;
-    }
-    a.vec = (n[0] & 1) == 0 && (((uintptr_t)phi_in | (uintptr_t)phi_out) & 15) == 0 &&
-            (((uintptr_t)pc_in | (uintptr_t)pc_out) & 31) == 0;
+    plan_columns(n, sm_count, &a);
+    a.vec = columns_vec(n[0], phi_in, phi_out, pc_in, pc_out);
     cudaError_t e = cudaFuncSetAttribute(column_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kColSmem);
     if (e != cudaSuccess) return e;
-    const dim3 grid((unsigned)gx, (unsigned)gy, (unsigned)((n[2] + a.zc - 1) / a.zc));
+    const dim3 grid((unsigned)((n[0] + a.vx - 1) / a.vx), (unsigned)((n[1] + a.vy - 1) / a.vy),
+                    (unsigned)((n[2] + a.zc - 1) / a.zc));
     column_kernel<<<grid, dim3(32, kColWarps), kColSmem, st>>>(a);
     return cudaGetLastError();
 }

@@ -21,7 +21,9 @@ cudaError_t launch_region(const RegionArgs &a, int threads, int B, int groups, s
 cudaError_t launch_sweep(const float2 *phi_in, float2 *phi_out, float4 *pc, const int n[3],
                          const LevelCoef *coef, int lvl, PhysConst q, cudaStream_t st);
 // Two levels of the whole grid in one pass, from one copy of the state to
-// another (sp_columns.cu); coef: of the first of them.
+// another (sp_columns.cu); coef: of the first of them.  columns_pay: whether
+// that is faster than two one-level sweeps of this grid.
+bool columns_pay(const float2 *phi, const float4 *pc, const int n[3], int sm_count);
 cudaError_t launch_columns(const float2 *phi_in, const float4 *pc_in, float2 *phi_out, float4 *pc_out, const int n[3],
                            const LevelCoef *coef, PhysConst q, int sm_count, cudaStream_t st);
 // Diagnostics of a stored state (sp_diag.cu): energy terms and winding counts
