@@ -1298,10 +1298,11 @@ int plan_lattice(sp_grid *g, const std::vector<int> &Bs, int threads)
         // places, 128 where the chain of layers counts (M^3 positions, 100 steps, us
         // with 64 / 128: edge 12, M = 6 744 / 564, 8 996 / 1085; edge 8 642 / 543,
         // 743 / 918).
-        long long layer_regions = 0;
-        for (int s = 0; s < g->n_sims; ++s)
-            layer_regions += 4ll * (g->p[s].n[0] / (4 * s_lat)) * (g->p[s].n[1] / (4 * s_lat)) * (g->p[s].n[2] / (4 * s_lat));
-        const bool few = s_lat >= 2 && layer_regions <= 7ll * g->sm_count;
+        long long per_layer = 0;  // of this launch's simulations
+        for (int sim = 0; sim < g->n_sims; ++sim)
+            if (g->B[sim] == c.B) per_layer += 4ll * (g->p[sim].n[0] / c.B) * (g->p[sim].n[1] / c.B) * (g->p[sim].n[2] / c.B);
+        if (per_layer > 0x7fffffffll) return SP_EINVAL;
+        const bool few = s_lat >= 2 && per_layer <= 7ll * g->sm_count;
         c.threads = threads ? threads : s_lat <= 3 && !few ? 64 : s_lat <= 4 ? 128 : s_lat == 5 ? 256 : 512;
         sp::LatConfig lc;
         e = sp::lattice_config(t, c.threads, &lc);
@@ -1312,10 +1313,6 @@ int plan_lattice(sp_grid *g, const std::vector<int> &Bs, int threads)
         c.grid = c.ctas_per_sm * g->sm_count;
         g->groups.push_back(c);
         g->lat_flag_off.push_back(flags);
-        long long per_layer = 0;
-        for (int sim = 0; sim < g->n_sims; ++sim)
-            if (g->B[sim] == c.B) per_layer += 4ll * (g->p[sim].n[0] / c.B) * (g->p[sim].n[1] / c.B) * (g->p[sim].n[2] / c.B);
-        if (per_layer > 0x7fffffffll) return SP_EINVAL;
         flags += 4 * (size_t)per_layer;
     }
     if ((int)g->groups.size() > kMaxGroups) return SP_EINVAL;
