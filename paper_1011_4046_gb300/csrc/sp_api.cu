@@ -68,6 +68,7 @@ struct LatOnDevice {
 struct GroupCfg {
     int B = 0, threads = 0, ctas_per_sm = 0, grid = 0;  // ctas_per_sm and grid count resident regions (base 32: CTAs)
     int groups = 1;                                     // regions per CTA
+    bool resident = false;                              // lattice: the kernel with the whole cell list
     size_t smem = 0;
 };
 
@@ -1086,7 +1087,7 @@ int evolve_lattice(sp_grid *g, int64_t n_steps, bool trace, bool timing)
         a.n_imp_run = (int)(t.imp_run.size() / 2);
         a.row_nb = ld.d_nb;
         a.row_pc = ld.d_pcoff;
-        a.cell_wide = reinterpret_cast<const uint2 *>(ld.d_wide);
+        a.cell_wide = c.resident ? reinterpret_cast<const uint2 *>(ld.d_wide) : nullptr;
         a.row_x0 = ld.d_row_x0;
         a.n_cell = (int)t.cell.size();
         a.groups = c.groups;
@@ -1305,10 +1306,11 @@ int plan_lattice(sp_grid *g, const std::vector<int> &Bs, int threads)
         const bool few = s_lat >= 2 && per_layer <= 7ll * g->sm_count;
         c.threads = threads ? threads : s_lat <= 3 && !few ? 64 : s_lat <= 4 ? 128 : s_lat == 5 ? 256 : 512;
         sp::LatConfig lc;
-        e = sp::lattice_config(t, c.threads, &lc);
+        e = sp::lattice_config(t, c.threads, per_layer <= 7ll * g->sm_count, &lc);
         if (e != cudaSuccess || lc.ctas_per_sm < 1) return SP_EINVAL;
         c.smem = lc.smem;
         c.groups = lc.groups;
+        c.resident = lc.resident;
         c.ctas_per_sm = lc.ctas_per_sm * lc.groups;
         c.grid = c.ctas_per_sm * g->sm_count;
         g->groups.push_back(c);

@@ -682,8 +682,7 @@ __global__ void lattice_reset_kernel(Ctl *ctl, int layers)
     lat_next_epoch(&ctl->last_layer, layers, &ctl->epoch);
 }
 
-// The kernel and its launch for a size: resident list (several regions per
-// CTA) where there are wide entries, else the ring.
+// The kernel of a size: resident list (several regions per CTA) or the ring.
 const void *lattice_fn(int threads, bool resident)
 {
     switch (threads) {
@@ -715,12 +714,25 @@ int lattice_max_groups(int threads)
 
 bool lattice_valid_threads(int threads) { return lattice_fn(threads, false) != nullptr; }
 
-cudaError_t lattice_config(const LatticeTables &t, int threads, LatConfig *c)
+// Whether a region per CTA with a ring of levels is the faster kernel although
+// the whole list fits: 64 workers at edges 16 and 20, whose 64 registers (16
+// regions of 64 threads would have to fit) cost the resident kernel more than the
+// shared list gives, at edge 12 where a layer has few regions, and 192 at edge 20,
+// where the list leaves room for two regions instead of three (32 steps, us,
+// resident / ring: edge 16, 64 workers, 128^3 728 / 641, 240^3 4601 / 4176; edge
+// 20, 64 workers, 160^3 2531 / 2229, 192 workers 1514 / 1441; edge 12, 64 workers,
+// 48^3 260 / 238, 240^3 4350 / 4939).  None of them is a default.
+bool lattice_ring_faster(int s, int threads, bool few)
+{
+    return (threads == 64 && (s >= 4 || (s == 3 && few))) || (threads == 192 && s >= 5);
+}
+
+cudaError_t lattice_config(const LatticeTables &t, int threads, bool few, LatConfig *c)
 {
     *c = LatConfig();
     if (!lattice_valid_threads(threads)) return cudaErrorInvalidValue;
     constexpr size_t kMost = 227 * 1024 - 2048;  // dynamic: the static arrays take up to 2 KB
-    const bool resident = !t.cell_wide.empty();
+    const bool resident = !t.cell_wide.empty() && !lattice_ring_faster(t.s, threads, few);
     const LatResident L((int)t.cell.size(), t.n_slots, t.n_foot, t.rb_side);
     const void *f = lattice_fn(threads, resident);
     // the number of regions per CTA that leaves the most of them on an SM
