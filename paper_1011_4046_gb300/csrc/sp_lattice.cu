@@ -149,12 +149,14 @@ __device__ __forceinline__ unsigned long long lat_site(int rx, unsigned yz, int 
 
 // A region's imports: the list of all of them (imp_run, in address order),
 // loaded in batches, of which a thread loads lat_imp_batch entries before using
-// any, so the entry reads overlap: with 128 workers 12 cover a whole region
-// of edge 16 (1370 entries) in one round of L2 latency.
+// any, so the entry reads overlap in one round of L2 latency: 12 cover a whole
+// region of edge 16 with 128 workers (1370 entries), 19 one of edge 20 with 256
+// (4609; 160^3, 4 steps 302 us, 328 with 12 in two rounds).  More than a size needs
+// costs code: edge 16 with 20 is 5 % slower.
 template <int NW>
 __host__ __device__ constexpr int lat_imp_batch()
 {
-    return NW == 64 ? 6 : NW == 192 ? 8 : 12;
+    return NW == 64 ? 6 : NW == 192 ? 8 : NW == 256 ? 19 : 12;
 }
 
 // One batch of import entries, i0 + u NW (padding: first level 255).
