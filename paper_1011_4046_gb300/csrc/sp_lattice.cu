@@ -292,7 +292,10 @@ __global__ void __launch_bounds__(lat_max_threads<NW>(), 1) lattice_kernel(const
     unsigned *const s_yz = reinterpret_cast<unsigned *>(mine + L.yz);
     LatRegion &s_reg = s_regs[group];
     volatile int &s_stop = s_stops[group], &s_next = s_nexts[group];
-    for (int i = threadIdx.x; i < a.n_cell; i += blockDim.x) s_cell[i] = a.cell_wide[i];
+    // the list by asynchronous copies, all on their way at once (an even number of
+    // 8-byte entries)
+    for (int i = 2 * threadIdx.x; i < a.n_cell; i += 2 * blockDim.x) cp_async16(s_cell + i, a.cell_wide + i);
+    cp_async_commit();
     for (int i = threadIdx.x; i < WW; i += blockDim.x) s_row_x0[i] = a.row_x0[i];
     for (int i = threadIdx.x; i <= a.K; i += blockDim.x) {
         s_cell_off[i] = a.cell_off[i];
@@ -313,6 +316,7 @@ __global__ void __launch_bounds__(lat_max_threads<NW>(), 1) lattice_kernel(const
     unsigned next = 0;
     int epoch = 0;
     int *unset = nullptr, unset_to = 0;  // flag of the finished region
+    cp_async_wait_all();
     __syncthreads();  // the shared lists; a region waits only after it: another group of the CTA may hold its predecessor
     const int bar = 1 + group;
     if (tid == ctl) {
