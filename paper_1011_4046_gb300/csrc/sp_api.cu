@@ -68,8 +68,12 @@ struct LatOnDevice {
 struct GroupCfg {
     int B = 0, threads = 0, ctas_per_sm = 0, grid = 0;  // ctas_per_sm and grid count resident regions (base 32: CTAs)
     int groups = 1;                                     // regions per CTA
-    bool resident = false;                              // lattice: the kernel with the whole cell list
     size_t smem = 0;
+    // lattice: the kernel with the whole cell list; and beside it, for calls of few
+    // steps, the launch of the kernel with a region per CTA (0 workers: none)
+    bool resident = false;
+    int brief_threads = 0, brief_grid = 0;
+    size_t brief_smem = 0;
 };
 
 // A group's launch in one call.
@@ -109,6 +113,13 @@ void append_key(std::vector<unsigned char> *key, const T &v)
 {
     const unsigned char *b = reinterpret_cast<const unsigned char *>(&v);
     key->insert(key->end(), b, b + sizeof(T));
+}
+
+// Member by member: the bytes between the members are anything.
+void append_key(std::vector<unsigned char> *key, const GroupCfg &c)
+{
+    for (const int v : {c.B, c.threads, c.ctas_per_sm, c.grid, c.groups, (int)c.resident}) append_key(key, v);
+    append_key(key, c.smem);
 }
 
 template <class T>
@@ -1087,10 +1098,17 @@ int evolve_lattice(sp_grid *g, int64_t n_steps, bool trace, bool timing)
         a.n_imp_run = (int)(t.imp_run.size() / 2);
         a.row_nb = ld.d_nb;
         a.row_pc = ld.d_pcoff;
-        a.cell_wide = c.resident ? reinterpret_cast<const uint2 *>(ld.d_wide) : nullptr;
+        if (c.brief_threads && sp::lattice_ring_brief(s, n_steps, per_layer_all, g->sm_count)) {
+            l.cfg.resident = false;
+            l.cfg.groups = 1;
+            l.cfg.threads = c.brief_threads;
+            l.cfg.smem = c.brief_smem;
+            l.cfg.grid = c.brief_grid;
+        }
+        a.cell_wide = l.cfg.resident ? reinterpret_cast<const uint2 *>(ld.d_wide) : nullptr;
         a.row_x0 = ld.d_row_x0;
         a.n_cell = (int)t.cell.size();
-        a.groups = c.groups;
+        a.groups = l.cfg.groups;
         a.bank_a = t.bank_a;
         a.bank_b = t.bank_b;
         a.max_cell_n = t.max_cell_n;
@@ -1306,8 +1324,17 @@ int plan_lattice(sp_grid *g, const std::vector<int> &Bs, int threads)
         const bool few = s_lat >= 2 && per_layer <= 7ll * g->sm_count;
         c.threads = threads ? threads : s_lat <= 3 && !few ? 64 : s_lat <= 4 ? 128 : s_lat == 5 ? 256 : 512;
         sp::LatConfig lc;
-        e = sp::lattice_config(t, c.threads, per_layer <= 7ll * g->sm_count, &lc);
+        e = sp::lattice_config(t, c.threads, sp::lattice_ring_faster(s_lat, c.threads, per_layer <= 7ll * g->sm_count), &lc);
         if (e != cudaSuccess || lc.ctas_per_sm < 1) return SP_EINVAL;
+        if (lc.resident && sp::lattice_ring_brief(s_lat, 1, per_layer, g->sm_count)) {
+            sp::LatConfig brief;
+            const int workers = threads ? threads : s_lat <= 2 ? 64 : 128;
+            e = sp::lattice_config(t, workers, true, &brief);
+            if (e != cudaSuccess || brief.ctas_per_sm < 1) return SP_EINVAL;
+            c.brief_threads = workers;
+            c.brief_smem = brief.smem;
+            c.brief_grid = brief.ctas_per_sm * g->sm_count;
+        }
         c.smem = lc.smem;
         c.groups = lc.groups;
         c.resident = lc.resident;

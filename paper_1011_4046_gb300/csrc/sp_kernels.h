@@ -60,7 +60,9 @@ struct LatConfig {
     size_t smem = 0;
 };
 bool lattice_valid_threads(int threads);
-cudaError_t lattice_config(const LatticeTables &t, int threads, bool few, LatConfig *c);  // few: regions of a layer
+bool lattice_ring_faster(int s, int threads, bool few);  // few: regions of a layer
+bool lattice_ring_brief(int s, long long n_steps, long long per_layer, int sms);
+cudaError_t lattice_config(const LatticeTables &t, int threads, bool ring, LatConfig *c);
 cudaError_t launch_lattice_reset(Ctl *ctl, int layers, cudaStream_t st);
 cudaError_t launch_lattice(const LatArgs &a, int threads, size_t smem, int grid, cudaStream_t st);
 }  // namespace sp

@@ -733,12 +733,27 @@ bool lattice_ring_faster(int s, int threads, bool few)
     return (threads == 64 && (s >= 4 || (s == 3 && few))) || (threads == 192 && s >= 5);
 }
 
-cudaError_t lattice_config(const LatticeTables &t, int threads, bool few, LatConfig *c)
+// The same for a call of few steps with 64 (s = 3: 128) workers: where a layer's
+// regions about fit the SMs, more of them are resident as CTAs of their own, and
+// no group waits its turn for a first ticket (resident / ring, us: edge 4, 32^3, 1
+// step 63 / 59, 8 steps 128 / 125; edge 8, 64^3, 1 step 69 / 63, 4 steps 87 / 82,
+// 8 steps 116 / 114, 16^3, 4 steps 49 / 58; edge 12, 72^3, 1 step 66 / 59, 8 steps
+// 102 / 97, 16 steps 144 / 139, 24^3, 8 steps 64 / 68, 96^3, 3 steps 104 / 98, 16
+// steps 237 / 242; beyond 14 regions per SM edge 4, 240^3 64 / 86 ms in 32 steps).
+bool lattice_ring_brief(int s, long long n_steps, long long per_layer, int sms)
+{
+    if (per_layer > 14ll * sms) return false;
+    if (s == 1) return n_steps <= 8;
+    if (per_layer <= 2ll * sms) return false;
+    return s == 2 ? n_steps <= 4 : s == 3 && n_steps <= (per_layer <= 7ll * sms ? 16 : 8);
+}
+
+cudaError_t lattice_config(const LatticeTables &t, int threads, bool ring, LatConfig *c)
 {
     *c = LatConfig();
     if (!lattice_valid_threads(threads)) return cudaErrorInvalidValue;
     constexpr size_t kMost = 227 * 1024 - 2048;  // dynamic: the static arrays take up to 2 KB
-    const bool resident = !t.cell_wide.empty() && !lattice_ring_faster(t.s, threads, few);
+    const bool resident = !t.cell_wide.empty() && !ring;
     const LatResident L((int)t.cell.size(), t.n_slots, t.n_foot, t.rb_side);
     const void *f = lattice_fn(threads, resident);
     // the number of regions per CTA that leaves the most of them on an SM
