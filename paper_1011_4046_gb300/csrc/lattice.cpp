@@ -370,18 +370,18 @@ std::string build_lattice_tables(int s, LatticeTables *t)
         // its site, per pair of imports in an even slot and the next one that
         // are x neighbours of one row
         const bool parity = (bank_a | bank_b) % 2 == 0;
-        std::map<std::pair<int, int>, size_t> at;  // (slot, buffer) -> index in imp_all
-        auto key = [&](size_t i) { return std::make_pair(lat_slot(t->imp_all[i]), (t->imp_all[i] & kLatImpBuf) ? 1 : 0); };
-        for (size_t i = 0; i < t->imp_all.size(); i += 2) at[key(i)] = i;
+        std::vector<int> at(2 * ((size_t)t->n_slots + 1), -1);  // slot and buffer -> index in imp_all
+        auto place = [&](uint32_t e, int slot) { return 2 * (size_t)slot + ((e & kLatImpBuf) ? 1 : 0); };
+        for (size_t i = 0; i < t->imp_all.size(); i += 2) at[place(t->imp_all[i], lat_slot(t->imp_all[i]))] = (int)i;
         size_t imports = 0;
         for (size_t i = 0; i < t->imp_all.size(); i += 2) {
             const uint32_t e = t->imp_all[i], k = t->imp_all[i + 1];
-            const auto other = at.find({lat_slot(e) ^ 1, key(i).second});
-            const bool pair = parity && (e & kLatImpPairRow) && other != at.end();
+            const int other = at[place(e, lat_slot(e) ^ 1)];
+            const bool pair = parity && (e & kLatImpPairRow) && other >= 0;
             if (pair && (lat_slot(e) & 1)) continue;  // in its lower neighbour's entry
             uint32_t w = k | k << 8;
             if (pair) {
-                const uint32_t e2 = t->imp_all[other->second], k2 = t->imp_all[other->second + 1];
+                const uint32_t e2 = t->imp_all[other], k2 = t->imp_all[other + 1];
                 if (lat_row(e2) != lat_row(e) || lat_rx2s(e2) != lat_rx2s(e) + 1) return fail("pair of imports not x neighbours");
                 w = std::min(k, k2) | std::max(k, k2) << 8 | kLatRunPair | ((e2 & kLatImpFull) ? kLatRunFull2 : 0u);
             }
