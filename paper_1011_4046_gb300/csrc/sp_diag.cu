@@ -35,6 +35,7 @@ struct DiagArgs {
     const float2 *phi;
     const float4 *pc;
     int nx, ny, nz, zc;
+    int flat;  // a block's threads are consecutive sites of a plane, not a 32 x 8 tile
     double eta2;
     float eta_w[3];  // eta^2 = eta_w[0] + [1] + [2], rounded words
     int fast;        // eta^2 in the range of the FP32 pairs
@@ -153,7 +154,12 @@ __global__ void __launch_bounds__(kDiagThreads, 3) diag_kernel(const DiagArgs a)
 {
     __shared__ double s_en[kDiagY][3];
     __shared__ int s_cnt[kDiagY][7];
-    const int x = blockIdx.x * 32 + threadIdx.x, y = blockIdx.y * kDiagY + threadIdx.y;
+    int x = blockIdx.x * 32 + threadIdx.x, y = blockIdx.y * kDiagY + threadIdx.y;
+    if (a.flat) {
+        x += (int)(blockIdx.x * (kDiagThreads - 32) + threadIdx.y * 32);
+        y = x / a.nx;
+        x -= y * a.nx;
+    }
     const int z0 = blockIdx.z * a.zc, z1 = min(z0 + a.zc, a.nz);
     const size_t plane = (size_t)a.nx * a.ny;
     const size_t sites = plane * a.nz;
@@ -326,9 +332,16 @@ __global__ void __launch_bounds__(256)
         out->winding[q - 3] = sl[0];
 }
 
+// Rows narrower than a warp would leave its lanes idle, of which a field that
+// needs the FP64 sums has none to spare: there a plane's sites go to the threads
+// one after the other (4 x 1024 x 1024, us, in tiles / so: 620 / 125, below the FP32
+// range 5530 / 1010; 16 x 512 x 512 199 / 124, 1856 / 954).
+bool diag_flat(int nx) { return nx < 32; }
+
 dim3 diag_grid(const int n[3], int *zc)
 {
     dim3 g((n[0] + 31) / 32, (n[1] + kDiagY - 1) / kDiagY, 1);
+    if (diag_flat(n[0])) g = dim3((n[0] * n[1] + kDiagThreads - 1) / kDiagThreads, 1, 1);
     // as many planes a thread as leave four blocks for every SM
     const long long cols = (long long)g.x * g.y;
     long long z = cols * n[2] / (4 * 152);
@@ -356,6 +369,7 @@ cudaError_t launch_diag(const float2 *phi, const float4 *pc, const int n[3], dou
     a.phi = phi;
     a.pc = pc;
     a.nx = n[0], a.ny = n[1], a.nz = n[2];
+    a.flat = diag_flat(n[0]);
     a.eta2 = eta2;
     a.fast = eta2 == 0.0 || (eta2 >= 0x1p-40 && eta2 <= 0x1p50);
     double r = a.fast ? eta2 : 0.0;
@@ -376,6 +390,7 @@ cudaError_t launch_winding_map(const float2 *phi, const int n[3], signed char *m
     const dim3 g = diag_grid(n, &a.zc);
     a.phi = phi;
     a.nx = n[0], a.ny = n[1], a.nz = n[2];
+    a.flat = diag_flat(n[0]);
     a.map = map;
     diag_kernel<false><<<g, dim3(32, kDiagY), 0, st>>>(a);
     return cudaGetLastError();
