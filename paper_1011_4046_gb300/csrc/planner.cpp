@@ -670,6 +670,44 @@ std::string build_octant_tables(const TileTables &t, OctTables *op)
     return std::string();
 }
 
+std::string build_preds(const TileTables &t, PredTables *p)
+{
+    p->preds.assign((size_t)2 * kTypes * kMaxPreds, Pred{{0, 0, 0}, 0});
+    for (int q = 0; q < 2; ++q)
+        for (int S = 0; S < kTypes; ++S) {
+            Pred *const out = p->preds.data() + (size_t)(q * kTypes + S) * kMaxPreds;
+            int n = 0;
+            bool phases = true;
+            auto add = [&](int type, int prev, const Succ &e) {
+                if (n < kMaxPreds) {
+                    out[n].type_prev = (unsigned char)(type | prev << 3);
+                    for (int d = 0; d < 3; ++d) out[n].e[d] = (signed char)-e.e[d];
+                }
+                ++n;
+            };
+            for (int from = 0; from < kTypes; ++from)
+                for (const Succ &e : t.same_succ[from])
+                    if (e.type == S) {
+                        phases = phases && __builtin_popcount((unsigned)from) < __builtin_popcount((unsigned)S);
+                        add(from, 0, e);
+                    }
+            p->n[S][0] = n;
+            for (const Succ &e : t.next_succ[q])
+                if (e.type == S) add(kTypes - 1, 1, e);
+            p->n[S][1] = n;
+            for (int from = 0; from < kTypes; ++from)
+                for (const Succ &e : t.reuse_succ[from])
+                    if (e.type == S) add(from, 1, e);
+            p->n[S][2] = n;
+            if (!phases) return "a same-band predecessor is not of an earlier phase";
+            if (p->n[S][0] != t.same_preds[S] || p->n[S][1] != t.same_preds[S] + t.prev_preds[S] ||
+                n != t.same_preds[S] + t.prev_preds[S] + t.reuse_preds[S])
+                return "predecessor counts differ from the planner's";
+            if (n > kMaxPreds) return "more predecessors than the table holds";
+        }
+    return std::string();
+}
+
 PlanStats plan_stats(const TileTables &t, const int n[3])
 {
     PlanStats s{};

@@ -157,6 +157,29 @@ std::string build_octant_tables(const TileTables &t, OctTables *o);
 // Returns an empty string on success or a description of the failed check.
 std::string build_tables(int B, TileTables *t);
 
+// The ticket order of a launch: bands in order, within a band the types by
+// number of inverted axes (kPhaseOrder, four bits each), within a type the
+// positions of all simulations.  A region waits for its predecessors, the
+// inverse of the successor patterns: the region of this type one band earlier
+// (prev) or in the same band, at the position offset e.
+constexpr unsigned kPhaseOrder = 0x76534210u;
+constexpr int kMaxPreds = 64;  // per type: two per lane of the manager warp
+struct Pred {
+    signed char e[3];
+    unsigned char type_prev;  // type | prev << 3
+};
+struct PredTables {
+    // by parity of the region's band and type, kMaxPreds each: the same band's,
+    // the previous band's, then those whose mailbox the region writes
+    std::vector<Pred> preds;
+    int32_t n[kTypes][3];  // of the first one, two, three kinds
+};
+
+// Builds them and checks what the ticket order relies on: a same-band
+// predecessor's type is of an earlier phase, and the counts are the planner's.
+// Returns an empty string on success.
+std::string build_preds(const TileTables &t, PredTables *p);
+
 // Region counts and HBM traffic for a whole grid at base B.
 struct PlanStats {
     int64_t regions_per_band, bands, updates_per_band;

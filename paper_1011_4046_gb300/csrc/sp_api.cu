@@ -347,50 +347,6 @@ int upload_reuse(const sp::TileTables &t, sp::Succ **d_reuse)
     return SP_OK;
 }
 
-// The predecessors of every type by parity of its band (the inverse of the
-// successor patterns), for the ticket order: the same band's, the previous
-// band's, those of mailbox reuse.  Checks what that order relies on: a
-// same-band predecessor's type is of an earlier phase, and the counts are the
-// planner's.
-int build_preds(const sp::TileTables &t, sp::TablesDev *h, std::vector<sp::Pred> *preds)
-{
-    preds->assign((size_t)2 * sp::kTypes * sp::kMaxPreds, sp::Pred{{0, 0, 0}, 0});
-    for (int q = 0; q < 2; ++q)
-        for (int S = 0; S < sp::kTypes; ++S) {
-            sp::Pred *out = preds->data() + (size_t)(q * sp::kTypes + S) * sp::kMaxPreds;
-            int n = 0;
-            bool ok = true;
-            auto add = [&](int type, int prev, const sp::Succ &e) {
-                if (n >= sp::kMaxPreds) {
-                    ok = false;
-                    return;
-                }
-                out[n].type_prev = (unsigned char)(type | prev << 3);
-                for (int d = 0; d < 3; ++d) out[n].e[d] = (signed char)-e.e[d];
-                ++n;
-            };
-            for (int from = 0; from < sp::kTypes; ++from)
-                for (const sp::Succ &e : t.same_succ[from])
-                    if (e.type == S) {
-                        ok = ok && __builtin_popcount((unsigned)from) < __builtin_popcount((unsigned)S);
-                        add(from, 0, e);
-                    }
-            ok = ok && n == t.same_preds[S];
-            h->pred_n[S][0] = (unsigned char)n;
-            for (const sp::Succ &e : t.next_succ[q])
-                if (e.type == S) add(sp::kTypes - 1, 1, e);
-            ok = ok && n == t.same_preds[S] + t.prev_preds[S];
-            h->pred_n[S][1] = (unsigned char)n;
-            for (int from = 0; from < sp::kTypes; ++from)
-                for (const sp::Succ &e : t.reuse_succ[from])
-                    if (e.type == S) add(from, 1, e);
-            ok = ok && n == t.same_preds[S] + t.prev_preds[S] + t.reuse_preds[S];
-            h->pred_n[S][2] = (unsigned char)n;
-            if (!ok) return SP_EINVAL;
-        }
-    return SP_OK;
-}
-
 // Base 32: the region's dependency pattern plus the octant tables of the
 // cluster kernel, packed for the device (see sp_device.cuh, TablesOct).
 int build_octant_device_tables(sp_grid *g, TablesOnDevice *tdp)
@@ -648,9 +604,11 @@ int build_device_tables(sp_grid *g, int B)
     up((void **)&td.d_imp, imp.data(), imp.size() * sizeof(unsigned short));
     up((void **)&td.d_exp, ex.data(), ex.size() * sizeof(int2));
     up((void **)&td.d_reuse, reuse.data(), reuse.size() * sizeof(sp::Succ));
-    std::vector<sp::Pred> preds;
-    if (build_preds(t, &h, &preds) != SP_OK) return SP_EINVAL;
-    up((void **)&td.d_preds, preds.data(), preds.size() * sizeof(sp::Pred));
+    sp::PredTables preds;
+    if (!sp::build_preds(t, &preds).empty()) return SP_EINVAL;
+    for (int S = 0; S < sp::kTypes; ++S)
+        for (int i = 0; i < 3; ++i) h.pred_n[S][i] = (unsigned char)preds.n[S][i];
+    up((void **)&td.d_preds, preds.preds.data(), preds.preds.size() * sizeof(sp::Pred));
     h.imp = td.d_imp;
     h.exp = td.d_exp;
     h.reuse = td.d_reuse;

@@ -54,14 +54,6 @@ struct alignas(16) TypeMeta {
     int n_reuse, reuse_preds;
 };
 
-// A predecessor of a region: the region of this type one band earlier (prev)
-// or in the same band, at the position offset e.
-struct Pred {
-    signed char e[3];
-    unsigned char type_prev;  // type | prev << 3
-};
-constexpr int kMaxPreds = 64;  // per type: two per lane of the manager warp
-
 // Geometry and surface-routing tables for one base size, in device memory.
 //
 // Import lists are 16-bit: a full-state import holds the cell's (pi, c) index

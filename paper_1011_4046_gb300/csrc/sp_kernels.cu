@@ -400,8 +400,6 @@ __device__ void manager_loop(const RegionArgs &a, const TablesDev *s_tabs, int *
     }
 }
 
-constexpr unsigned kPhaseOrder = 0x76534210u;  // the region types by number of inverted axes
-
 // The region of ticket t: bands in order, within a band the types by phase (a
 // predecessor's type is a subset of the region's, one phase or more earlier),
 // within a type the positions of all simulations.  Region ids stay those of
