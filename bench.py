@@ -66,9 +66,9 @@ SAMPLE_Z = 32
 # band-top state plus sloped faces, counted by brute force over one
 # steady-state band (each face cell written once, read by every consumer).
 ALG_BYTES_PER_UPDATE = {8: 42.8, 16: 25.3, 32: 13.8}
-# The whole-grid sweep takes two levels per pass over phi (8 B) and (pi, c)
-# (16 B), each read and written once.
-MONO_BYTES_PER_UPDATE = 24.0
+# The whole-grid sweep reads and writes phi (8 B) and (pi, c) (16 B) once per
+# level, or, where it takes two levels per pass, once per two.
+MONO_BYTES_PER_UPDATE = 48.0
 # On-chip (shared-memory) bytes per site-update of the region kernel: seven
 # phi reads (8 B) and one phi write, one (pi, c) read and write (16 B each).
 SMEM_BYTES_PER_UPDATE = 7 * 8 + 8 + 2 * 16
@@ -89,6 +89,15 @@ def workload_name(w):
                else f"region base B={w['B']}")
     return (f"{n}^3 matter era (nu=2, tau0=10, tau_ref={TAU0 + steps * DT:g}), lambda=2, eta=1, dx=1, dt=0.25, "
             f"random-phase init seed 0, {steps} leapfrog steps, {regions}")
+
+
+def sweep_bytes_per_update(sites, steps, taken):
+    """HBM bytes per site-update of a sweep call of `steps` levels whose handle
+    holds `taken` bytes of scratch: a copy of phi (8 B a site), and of (pi, c)
+    (16 B) as well where the call takes two levels per pass, which it does for
+    all but the last steps mod 4."""
+    pairs = steps // 4 * 4 if taken >= 20 * sites else 0
+    return MONO_BYTES_PER_UPDATE * (1.0 - 0.5 * pairs / steps)
 
 
 def lattice_layers(B, steps):
@@ -470,6 +479,7 @@ def run_grid(args, w, extra=None):
         phi.copy_(phi0)
         pic.zero_()
         gm = sp.Grid([p], states=[(phi, pic)], stream=stream)
+        free_before = torch.cuda.mem_get_info()[0]
         try:
             gm.set_level(0, restore_level)
             ms = []
@@ -484,12 +494,14 @@ def run_grid(args, w, extra=None):
                 e1.synchronize()
                 if it:
                     ms.append(e0.elapsed_time(e1))
+            sweep_bytes = sweep_bytes_per_update(N ** 3, PER, free_before - torch.cuda.mem_get_info()[0])
         finally:
             gm.close()
         mv = updates * len(ms) / (sum(ms) / 1e3)
         mono = {"value": mv, "unit": "site-updates/s", "ms_per_step": sum(ms) / len(ms), "steps": len(ms),
                 "speedup_of_regions": value / ws / mv,
-                "roofline_frac": MONO_BYTES_PER_UPDATE * mv / 1e9 / peaks()[0]}
+                "bytes_per_update": sweep_bytes,
+                "roofline_frac": sweep_bytes * mv / 1e9 / peaks()[0]}
     del phi, pic, phi0
     torch.cuda.empty_cache()
 
