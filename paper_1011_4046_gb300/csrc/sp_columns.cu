@@ -19,8 +19,8 @@
 // 1 a thread keeps the planes p - 1 .. p - 3 of phi and p - 1, p - 2 of (pi, c)
 // in registers; x neighbours come by shuffles, the rows above and below the
 // warp's two through shared memory.  Input planes arrive by cp.async two steps
-// ahead.  Why this tile: 15 warps of two rows use 127 registers a thread and
-// 167 KB of shared memory, one CTA per SM; at 512^3 other shapes measured
+// ahead.  Why this tile: 15 warps of two rows use 124 registers a thread and
+// 200 KB of shared memory, one CTA per SM; at 512^3 other shapes measured
 // 1.12 ms (32 rows), 1.13 (two CTAs of 16 rows), 1.18 (24), 1.23 (24 rows, one
 // row per warp).  Three and four levels a pass move less but spill or leave
 // too few warps for the longer chain: 1.63 ms (three levels, 2.47e11) and 2.44

@@ -7,7 +7,8 @@
 // 1278 phi slots in each of two parity buffers and 878 (pi, c) slots, 34.5
 // KB), so several regions run on one SM: as groups of threads of one CTA that
 // shares the cell list (lattice_kernel, up to edge 20; five at s = 4), or one
-// per CTA (lattice_ring_kernel, edge 24, whose list does not fit).  A region
+// per CTA (lattice_ring_kernel: edge 24, whose list does not fit, and the worker
+// counts and short calls of lattice_ring_faster and lattice_ring_brief).  A region
 //   1. waits until its four predecessors (layer L - 1) have reported done,
 //   2. copies in the values it does not compute (cp.async: phi of the halo
 //      and the whole state of cells entering the region), straight from the
@@ -23,12 +24,14 @@
 // every region.  A site index follows from the cell's slot and row through the
 // row's wrapped y + n1 z, which is refilled for each region, without a branch.
 //
-// Regions are handed out by ticket in layer order (one atomic per region,
-// taken a region ahead; the next region's predecessor flags are read early,
-// relaxed, and one fence per region serves as the release of its writes and
-// the acquire of those reads).  A ticket's predecessors hold smaller tickets, and
-// a group holding a ticket is running or will run it next, so the waits always
-// end; each is bounded anyway.  The manager of the paper (Sec. 4) is thus
+// Regions are handed out by ticket in layer order (one atomic per region, taken
+// a region ahead).  In lattice_kernel a region's flag is set by a releasing store
+// and the next region's flags are read by acquiring loads, both while the next
+// region's imports are on their way; in lattice_ring_kernel the flags are read
+// early, relaxed, and one fence per region serves as the release of its writes
+// and the acquire of those reads.  A ticket's predecessors hold smaller tickets,
+// and a group holding a ticket is running or will run it next, so the waits
+// always end; each is bounded anyway.  The manager of the paper (Sec. 4) is thus
 // reduced to a counter and one flag per region.
 #include <cuda_runtime.h>
 #include <stdint.h>
@@ -151,8 +154,8 @@ __device__ __forceinline__ unsigned long long lat_site(int rx, unsigned yz, int 
 // loaded in batches, of which a thread loads lat_imp_batch entries before using
 // any, so the entry reads overlap in one round of L2 latency: 12 cover a whole
 // region of edge 16 with 128 workers (1370 entries), 19 one of edge 20 with 256
-// (4609; 160^3, 4 steps 302 us, 328 with 12 in two rounds).  More than a size needs
-// costs code: edge 16 with 20 is 5 % slower.
+// (4609; 240^3, 32 steps 4079 us with 12 in two rounds, 3832 so; 160^3, 4 steps 331
+// and 301).  More than a size needs costs code: edge 16 with 20 is 5 % slower.
 template <int NW>
 __host__ __device__ constexpr int lat_imp_batch()
 {
@@ -310,7 +313,7 @@ __global__ void __launch_bounds__(lat_max_threads<NW>(), 1) lattice_kernel(const
     // regions than the GPU holds, the region follows without a wait, a fence or a
     // barrier of its own (with a fence, the flag and the early reads' check between
     // two regions: edge 16 1.390e11 site-updates/s at 240^3, now 1.449e11; edge 8
-    // 0.534 and 0.588e11; edge 20 1.121 and 1.205e11).
+    // 0.534 and 0.588e11; edge 20 1.121 and 1.205e11, with imports in two rounds).
     const int ctl = NW - 1;
     const bool ctl_warp = tid >= NW - 32;
     unsigned next = 0;
@@ -471,7 +474,7 @@ __global__ void __launch_bounds__(lat_max_threads<NW>(), 1) lattice_kernel(const
     }
 }
 
-// ---- the kernel for larger sizes: a region per CTA, a ring of two levels' entries ----
+// ---- the kernel with a region per CTA and a ring of two levels' entries ----
 // (a level's cell entries are copied into shared memory a level ahead; a cell's
 // neighbours, (pi, c) slot and site index follow from its slot and a 16-byte
 // record of its row)
