@@ -1272,17 +1272,17 @@ int plan_lattice(sp_grid *g, const std::vector<int> &Bs, int threads)
         // 0.91e11, 192: 1.21e11), 256 at s = 5, 512 at s = 6
         const int s_lat = it->first;
         // Edges 8 and 12 take 64 workers where a layer has regions for every SM's
-        // places, 128 where the chain of layers counts (M^3 positions, 100 steps, us
-        // with 64 / 128: edge 12, M = 6 744 / 564, 8 996 / 1085; edge 8 642 / 543,
-        // 743 / 918).
+        // places, 128 where the chain of layers counts (regions per SM, us with 64 /
+        // 128: edge 12, 91 steps, 6.6 676 / 583, 9.0 793 / 735, 10.3 841 / 799, 11.8 879 /
+        // 886, 13.5 971 / 1001; edge 8 5.7 593 / 560, 6.6 603 / 612, 9.0 626 / 655).
         long long per_layer = 0;  // of this launch's simulations
         for (int sim = 0; sim < g->n_sims; ++sim)
             if (g->B[sim] == c.B) per_layer += 4ll * (g->p[sim].n[0] / c.B) * (g->p[sim].n[1] / c.B) * (g->p[sim].n[2] / c.B);
         if (per_layer > 0x7fffffffll) return SP_EINVAL;
-        const bool few = s_lat >= 2 && per_layer <= 7ll * g->sm_count;
+        const bool few = per_layer <= (s_lat == 2 ? 6ll : s_lat == 3 ? 11ll : 0ll) * g->sm_count;
         c.threads = threads ? threads : s_lat <= 3 && !few ? 64 : s_lat <= 4 ? 128 : s_lat == 5 ? 256 : 512;
         sp::LatConfig lc;
-        e = sp::lattice_config(t, c.threads, sp::lattice_ring_faster(s_lat, c.threads, per_layer <= 7ll * g->sm_count), &lc);
+        e = sp::lattice_config(t, c.threads, sp::lattice_ring_faster(s_lat, c.threads, per_layer <= 12ll * g->sm_count), &lc);
         if (e != cudaSuccess || lc.ctas_per_sm < 1) return SP_EINVAL;
         if (lc.resident && sp::lattice_ring_brief(s_lat, 1, per_layer, g->sm_count)) {
             sp::LatConfig brief;

@@ -726,11 +726,12 @@ bool lattice_valid_threads(int threads) { return lattice_fn(threads, false) != n
 // Whether a region per CTA with a ring of levels is the faster kernel although
 // the whole list fits: 64 workers at edges 16 and 20, whose 64 registers (16
 // regions of 64 threads would have to fit) cost the resident kernel more than the
-// shared list gives, at edge 12 where a layer has few regions, and 192 at edge 20,
+// shared list gives, at edge 12 up to 12 regions of a layer per SM, and 192 at edge 20,
 // where the list leaves room for two regions instead of three (32 steps, us,
 // resident / ring: edge 16, 64 workers, 128^3 728 / 641, 240^3 4601 / 4176; edge
 // 20, 64 workers, 160^3 2531 / 2229, 192 workers 1514 / 1441; edge 12, 64 workers,
-// 48^3 260 / 238, 240^3 4350 / 4939).  None of them is a default.
+// 48^3 260 / 238, 84^3, 91 steps 799 / 703, 240^3 4350 / 4939).  None of them is a
+// default.
 bool lattice_ring_faster(int s, int threads, bool few)
 {
     return (threads == 64 && (s >= 4 || (s == 3 && few))) || (threads == 192 && s >= 5);
@@ -740,7 +741,7 @@ bool lattice_ring_faster(int s, int threads, bool few)
 // regions about fit the SMs, more of them are resident as CTAs of their own, and
 // no group waits its turn for a first ticket (resident / ring, us: edge 4, 32^3, 1
 // step 63 / 59, 8 steps 128 / 125; edge 8, 64^3, 1 step 69 / 63, 4 steps 87 / 82,
-// 8 steps 116 / 114, 16^3, 4 steps 49 / 58; edge 12, 72^3, 1 step 66 / 59, 8 steps
+// 8 steps 116 / 114, 56^3, 8 steps 106 / 95, 48^3, 6 steps 84 / 84, 16^3, 4 steps 49 / 58; edge 12, 72^3, 1 step 66 / 59, 8 steps
 // 102 / 97, 16 steps 144 / 139, 24^3, 8 steps 64 / 68, 96^3, 3 steps 104 / 98, 16
 // steps 237 / 242; beyond 14 regions per SM edge 4, 240^3 64 / 86 ms in 32 steps).
 bool lattice_ring_brief(int s, long long n_steps, long long per_layer, int sms)
@@ -748,7 +749,7 @@ bool lattice_ring_brief(int s, long long n_steps, long long per_layer, int sms)
     if (per_layer > 14ll * sms) return false;
     if (s == 1) return n_steps <= 8;
     if (per_layer <= 2ll * sms) return false;
-    return s == 2 ? n_steps <= 4 : s == 3 && n_steps <= (per_layer <= 7ll * sms ? 16 : 8);
+    return s == 2 ? n_steps <= (per_layer <= 6ll * sms ? 4 : 8) : s == 3 && n_steps <= (per_layer <= 7ll * sms ? 16 : 8);
 }
 
 cudaError_t lattice_config(const LatticeTables &t, int threads, bool ring, LatConfig *c)
