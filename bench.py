@@ -779,7 +779,7 @@ def main():
     ap.add_argument("--shape", default=None, choices=["split", "lattice"],
                     help="region geometry: the paper's 4-cube lattice or the split tiling (pyramids and "
                          "wedges); default: the lattice for the grid workloads, the split tiling for the "
-                         "batch (each measured the faster there)")
+                         "batch")
     ap.add_argument("--threads", type=int, default=0, help="threads per CTA (0 = library default)")
     ap.add_argument("--grid", type=int, default=0, help="grid side (profiling of smaller cases only)")
     ap.add_argument("--per-step", type=int, default=0, help="leapfrog steps per bench step (profiling only)")
