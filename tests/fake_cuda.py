@@ -9,7 +9,6 @@ import subprocess
 from paper_1011_4046_gb300 import build, sp
 
 HERE = os.path.dirname(os.path.abspath(__file__))
-CUDA_INCLUDE = os.path.join(os.path.dirname(os.path.dirname(build.nvcc())), "include")
 
 
 def load():
@@ -21,7 +20,8 @@ def load():
     objs = sorted(o for o in glob.glob(os.path.join(build.BUILD, "*.o")) if os.path.basename(o)[:-2] in build.SOURCES)
     if not os.path.exists(lib) or any(os.path.getmtime(f) > os.path.getmtime(lib) for f in [src, *objs]):
         tmp = lib + f".tmp{os.getpid()}"
-        subprocess.run(["g++", "-O1", "-std=c++17", "-fPIC", "-shared", f"-I{CUDA_INCLUDE}", src, *objs,
+        include = os.path.join(os.path.dirname(os.path.dirname(build.nvcc())), "include")
+        subprocess.run(["g++", "-O1", "-std=c++17", "-fPIC", "-shared", f"-I{include}", src, *objs,
                         "-Wl,-Bsymbolic", "-Wl,-z,defs", "-o", tmp], check=True)
         os.replace(tmp, lib)
     L = ctypes.CDLL(lib)
