@@ -12,7 +12,7 @@ HERE = os.path.dirname(os.path.abspath(__file__))
 
 
 def load():
-    build.build()
+    build.build(force=not all(os.path.exists(os.path.join(build.BUILD, f + ".o")) for f in build.SOURCES))
     out_dir = os.path.join(HERE, "cpu_exec", "_build")
     os.makedirs(out_dir, exist_ok=True)
     lib = os.path.join(out_dir, "libsp_fake.so")
